@@ -239,8 +239,8 @@ typedef struct {
    wall halo at the domain faces; FP64 cases run the generic sweep kernel.
    Cases with a wall cannot be batch members.  The state is kept.  With any wall the library allocates
    (2 ncell / n[a] summed over the D axes) * nvel_padded * ncomp elements of
-   the storage type for the halo values, and frees them with the context or
-   on the next call.
+   the storage type for the halo values and 6 nvel_padded doubles for the walls'
+   Maxwellians, and frees them with the context or on the next call.
    Errors: IBDVM_E_INVAL (a bad kind, a z wall in 2D, T_w <= 0 or a
    non-finite U_w; nothing changes), IBDVM_E_STATE (the context is a batch
    member), IBDVM_E_NOMEM. */

@@ -93,6 +93,40 @@ template <typename T> std::vector<T> cast(const std::vector<double> &v) {
   return std::vector<T>(v.begin(), v.end());
 }
 
+// per face and stored velocity of diffuse domain walls: the weight w |xi_a| of
+// the mass flux out of the domain, or, for velocities entering it, minus the
+// unit-density wall Maxwellian (Eq. boundary maxwell; the sign bit marks them
+// even where it underflows); in[face] receives that Maxwellian's mass flux
+std::vector<double> wall_table(const ibdvm_ctx *ctx, const ibdvm_domain_desc &d, int mask, double in[6]) {
+  const Geom &G = ctx->geom;
+  const size_t nvp = ctx->nvp;
+  std::vector<double> t(6 * nvp, 0.0);
+  for (int i = 0; i < 6; ++i) {
+    in[i] = 0.0;
+    if (!(mask >> i & 1)) continue;
+    const int a = i >> 1;
+    const double s = (i & 1) ? 1.0 : -1.0, Tw = d.T_w[i];
+    const double norm = (G.dim == 2) ? 1.0 / (kPi * Tw) : 1.0 / std::pow(kPi * Tw, 1.5);
+    for (int k = 0; k < G.nv; ++k) {
+      const double xs = s * G.xi[3 * k + a];
+      double &e = t[i * nvp + ctx->kst_h[k]];
+      if (!(xs < 0.0)) {
+        e = std::fabs(G.w[k] * xs); // 0, not -0, for a zero component
+        continue;
+      }
+      double c2 = 0.0;
+      for (int b = 0; b < G.dim; ++b) {
+        const double c = G.xi[3 * k + b] - d.U_w[i][b];
+        c2 += c * c;
+      }
+      const double M = norm * std::exp(-c2 / Tw);
+      in[i] += G.w[k] * xs * M;
+      e = -M;
+    }
+  }
+  return t;
+}
+
 void free_body(ibdvm_ctx *ctx) {
   void *ps[] = {ctx->dslot, ctx->dlinks, ctx->l_int, ctx->l_dbl, ctx->l_wg, ctx->g_int, ctx->s_int,
                 ctx->s_dbl, ctx->lval, ctx->fi_scr, ctx->fsp_scr, ctx->rhow, ctx->fpart, ctx->gw_unit};
@@ -141,6 +175,7 @@ void free_all(ibdvm_ctx *ctx) {
   cfree_t(ctx->d_forces);
   cfree_t(ctx->d_step_forces);
   cfree(ctx->whalo);
+  cfree(ctx->wall_tab);
   for (cudaEvent_t &e : ctx->copy_ev)
     if (e) {
       cudaEventDestroy(e);
@@ -903,26 +938,48 @@ ibdvm_status ibdvm_set_domain(ibdvm_ctx *ctx, const ibdvm_domain_desc *d) {
   const Geom &G = ctx->geom;
   long long off[7] = {};
   for (int i = 0; i < 6; ++i) off[i + 1] = off[i] + ((i < 2 * D) ? ctx->ncell / G.n[i >> 1] : 0);
-  void *halo = nullptr;
+  const size_t halo_bytes = static_cast<size_t>(off[6]) * ctx->nvp * ctx->ncomp * ctx->esize;
+  const size_t tab_bytes = 6 * static_cast<size_t>(ctx->nvp) * sizeof(double);
+  void *halo = nullptr, *tab = nullptr;
+  double in[6] = {};
   if (mask) {
-    const size_t bytes = static_cast<size_t>(off[6]) * ctx->nvp * ctx->ncomp * ctx->esize;
-    if (cudaMalloc(&halo, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      ctx->err = "set_domain: device allocation of the wall halo (" + std::to_string(bytes) + " bytes) failed";
-      return IBDVM_E_NOMEM;
+    const std::vector<double> t = wall_table(ctx, *d, mask, in);
+    std::vector<float> t2; // FP32 storage: every entry as the sum of two floats
+    if (ctx->precision != IBDVM_FP64) {
+      t2.resize(2 * t.size());
+      for (size_t k = 0; k < t.size(); ++k) {
+        t2[2 * k] = static_cast<float>(t[k]);
+        t2[2 * k + 1] = static_cast<float>(t[k] - static_cast<double>(t2[2 * k]));
+      }
     }
-    ctx->dev_bytes += bytes;
+    const void *src = t2.empty() ? static_cast<const void *>(t.data()) : t2.data();
+    const bool ok = cudaMalloc(&halo, halo_bytes) == cudaSuccess && cudaMalloc(&tab, tab_bytes) == cudaSuccess;
+    cudaError_t e = ok ? cudaMemcpyAsync(tab, src, tab_bytes, cudaMemcpyHostToDevice, ctx->stream) : cudaSuccess;
+    if (ok && e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream); // the host table goes out of scope
+    if (!ok || e != cudaSuccess) {
+      cudaGetLastError();
+      if (halo) cudaFree(halo);
+      if (tab) cudaFree(tab);
+      ctx->err = ok ? std::string("set_domain: upload of the wall table: ") + cudaGetErrorString(e)
+                    : "set_domain: device allocation of the wall halo (" + std::to_string(halo_bytes + tab_bytes) +
+                          " bytes) failed";
+      return ok ? IBDVM_E_CUDA : IBDVM_E_NOMEM;
+    }
+    ctx->dev_bytes += halo_bytes + tab_bytes;
   }
   if (ctx->whalo) {
     sync(ctx, "drain before replacing the wall halo");
     cudaFree(ctx->whalo);
-    ctx->dev_bytes -= static_cast<size_t>(ctx->wall_off[6]) * ctx->nvp * ctx->ncomp * ctx->esize;
+    cudaFree(ctx->wall_tab);
+    ctx->dev_bytes -= static_cast<size_t>(ctx->wall_off[6]) * ctx->nvp * ctx->ncomp * ctx->esize + tab_bytes;
   }
   ctx->whalo = halo;
+  ctx->wall_tab = tab;
   ctx->wall_mask = mask;
   for (int i = 0; i < 7; ++i) ctx->wall_off[i] = mask ? off[i] : 0;
   for (int i = 0; i < 6; ++i) {
     ctx->wall_T[i] = (mask >> i & 1) ? d->T_w[i] : 1.0;
+    ctx->wall_in[i] = in[i];
     for (int a = 0; a < 3; ++a) ctx->wall_U[i][a] = (mask >> i & 1) ? d->U_w[i][a] : 0.0;
   }
   // the TMA sweeps read the wall halo at the domain faces

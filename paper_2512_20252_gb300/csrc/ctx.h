@@ -123,6 +123,11 @@ struct ibdvm_ctx {
   double wall_U[6][3] = {};
   long long wall_off[7] = {};
   void *whalo = nullptr;
+  // per face and stored velocity, the weight of the mass flux out of the
+  // domain or minus the unit-density wall Maxwellian ([6][nvp] of double, or
+  // of two floats for FP32 storage), and the mass flux of that Maxwellian
+  void *wall_tab = nullptr;
+  double wall_in[6] = {};
   bool tma_ok = false; // the TMA sweep was set up (it serves cases with and without domain walls)
   // a tree-refined 2D grid: the cells are the leaves of a quadtree
   bool tree = false;

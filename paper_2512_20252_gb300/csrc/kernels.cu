@@ -1554,83 +1554,142 @@ __global__ void __launch_bounds__(kGhostThreads, (GhostTiling<T, false>::blocks)
 // diffuse domain walls: the halo values of every boundary cell of a wall face
 // ---------------------------------------------------------------------------
 
+// The wall's part in a value, tabulated per face and velocity when the walls
+// are set (wall_table): for velocities leaving the domain the weight w |xi_a|
+// of their mass flux, for the entering ones minus the unit-density wall
+// Maxwellian (the sign bit marks them).  FP32 storage keeps the FP64 entry as
+// the sum of two FP32 values.
+template <typename T> struct WallEntry;
+template <> struct WallEntry<double> { using type = double; };
+template <> struct WallEntry<float> { using type = float2; };
+
 template <typename T> struct DomainArgs {
   const T *__restrict__ f;
   const uint8_t *__restrict__ ctype;
-  const double *__restrict__ xiD; // [3][nvp]
-  const double *__restrict__ wD;  // [nvp]
+  const typename WallEntry<T>::type *__restrict__ tab; // [6][nvp]
   T *__restrict__ whalo;          // [slots][nvp][NC]
-  const int *__restrict__ kst;    // [nv] stored position of each velocity (natural order)
   long long off[7];               // first slot of each face; off[6] = all slots
-  int mask;
+  int grp[7];                     // first block of each face (S slots each, none for a freestream face)
   int n[3];
-  int nv, nvp;
-  double Tw[6], Uw[6][3];
+  int nvp;
+  double in[6];                   // unit-density wall mass flux into the domain (negative)
+  double halfT[6];                // T_w / 2
 };
 
 constexpr int kDomainThreads = 256;
+// boundary cells of one block: they share the table reads, but a face of few
+// cells needs every block it can give (below kDomainFew cells one per block:
+// 256 cells of 64^2 with 100^2 velocities 39 us against 76 us with four)
+constexpr int kDomainSlots = 4;
+constexpr int kDomainFew = 8 * 152;
 
-// One block per slot of a wall face: the boundary cell's mass flux out of the
-// domain through the face, carried by its own value (sum over s xi_a > 0), is
-// returned by rho_w times the face's unit-density wall Maxwellian (the plane
-// xi_a = 0 splits the velocities; FP64 sums); the halo then holds rho_w M_w
-// for the entering velocities and the cell's own value for the others.
-template <typename T, int D> __global__ void __launch_bounds__(kDomainThreads) domain_wall_kernel(DomainArgs<T> A) {
+// Sum of products c f in FP32 storage to nearly twice FP32's precision: the
+// rounding errors of the product (by FMA) and of the sum (Knuth's TwoSum) are
+// summed beside it (Ogita, Rump and Oishi's Dot2).  GB300 has 2 FP64 lanes per
+// clock and SM against 128 FP32 lanes, so this costs a fraction of one FP64 FMA.
+__device__ __forceinline__ void dot2(float &s, float &e, float2 c, float f) {
+  const float p = __fmul_rn(c.x, f);
+  const float ep = __fmaf_rn(c.y, f, __fmaf_rn(c.x, f, -p));
+  const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+  e += __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z)), ep);
+  s = t;
+}
+__device__ __forceinline__ void dot2(double &s, double &, double c, double f) { s += c * f; }
+// rho M of a wall density split into two values and a table entry
+__device__ __forceinline__ float wall_value(float2 r, float2 m) {
+  const float p = __fmul_rn(r.x, m.x);
+  return __fadd_rn(p, __fmaf_rn(r.x, m.y, __fmaf_rn(r.y, m.x, __fmaf_rn(r.x, m.x, -p))));
+}
+__device__ __forceinline__ double wall_value(double r, double m) { return r * m; }
+__device__ __forceinline__ bool entering(float2 c) { return signbit(c.x); }
+__device__ __forceinline__ bool entering(double c) { return signbit(c); }
+__device__ __forceinline__ void split(double v, double &o) { o = v; }
+__device__ __forceinline__ void split(double v, float2 &o) {
+  o.x = (float)v;
+  o.y = (float)(v - (double)o.x);
+}
+
+// One block per S slots of a wall face: each boundary cell's mass
+// flux out of the domain through the face, carried by its own values (sum over
+// s xi_a > 0), is returned by rho_w times the face's unit-density wall
+// Maxwellian (the plane xi_a = 0 splits the velocities); the halo then holds
+// rho_w M_w for the entering velocities and the cell's own value for the
+// others.  f is read once and the halo written once; the wall Maxwellian and
+// the flux weights come from a table (L2).  Closed box of 32^3 cells and 16^3
+// velocities, FP32: 80 us per step, where forming the Maxwellian per value in
+// FP64, twice, had taken 2487 us; 64^2 cells and 100^2 velocities: 39 us (265).
+template <typename T, int D, int S>
+__global__ void __launch_bounds__(kDomainThreads) domain_wall_kernel(DomainArgs<T> A) {
   constexpr int NC = Dims<D>::NC;
-  __shared__ double sh[kDomainThreads / 32 + 1];
-  const long long slot = blockIdx.x;
+  using E = typename WallEntry<T>::type;
+  __shared__ double sh[S][kDomainThreads / 32];
+  __shared__ E s_rho[2][S]; // rho_w, and T_w / 2 rho_w
   int i = 0;
-  while (i < 5 && slot >= A.off[i + 1]) ++i;
-  if (!((A.mask >> i) & 1)) return; // a freestream face: no slots in use
+  while (i < 5 && (int)blockIdx.x >= A.grp[i + 1]) ++i;
   const int a = i >> 1, s = (i & 1) ? 1 : -1;
-  const long long t = slot - A.off[i];
-  int ijk[3];
   const int u = (a == 0) ? 1 : 0, v = (a == 2) ? 1 : 2; // the transverse axes, in order
-  ijk[a] = (s > 0) ? A.n[a] - 1 : 0;
-  ijk[u] = (int)(t % A.n[u]);
-  ijk[v] = (int)(t / A.n[u]);
-  const long long c = ijk[0] + (long long)A.n[0] * (ijk[1] + (long long)A.n[1] * ijk[2]);
-  T *dst = A.whalo + (size_t)slot * A.nvp * NC;
-  const T *fc = A.f + (size_t)c * A.nvp * NC;
-  if (A.ctype[c] != IBDVM_CELL_FLUID) { // never read: the cell has no faces of its own
-    for (int k = threadIdx.x; k < A.nvp * NC; k += blockDim.x) dst[k] = T(0);
-    return;
-  }
-  const double Tw = A.Tw[i];
-  const double norm = (D == 2) ? 1.0 / (kPi * Tw) : 1.0 / pow(kPi * Tw, 1.5);
-  double so = 0.0, si = 0.0;
-  for (int iv = threadIdx.x; iv < A.nv; iv += blockDim.x) {
-    const int k = A.kst[iv];
-    const double xs = s * A.xiD[a * A.nvp + k];
-    if (xs > 0.0) {
-      so += A.wD[k] * xs * (double)fc[(size_t)k * NC];
-    } else if (xs < 0.0) {
-      double c2 = 0.0;
-      for (int b = 0; b < D; ++b) {
-        const double cb = A.xiD[b * A.nvp + k] - A.Uw[i][b];
-        c2 += cb * cb;
-      }
-      si += A.wD[k] * xs * norm * exp(-c2 / Tw);
-    }
-  }
-  const double out = block_sum<kDomainThreads>(so, sh);
-  const double in = block_sum<kDomainThreads>(si, sh);
-  const double rho_w = -out / in;
-  for (int k = threadIdx.x; k < A.nvp; k += blockDim.x) {
-    const double xs = s * A.xiD[a * A.nvp + k]; // zero at padding positions
-    if (xs < 0.0) {
-      double c2 = 0.0;
-      for (int b = 0; b < D; ++b) {
-        const double cb = A.xiD[b * A.nvp + k] - A.Uw[i][b];
-        c2 += cb * cb;
-      }
-      const double H = rho_w * norm * exp(-c2 / Tw);
-      dst[(size_t)k * NC] = (T)H;
-      if (NC == 2) dst[(size_t)k * NC + NC - 1] = (T)(0.5 * Tw * H); // B_w = T_w / 2 H_w
-    } else {
+  const long long t0 = (long long)((int)blockIdx.x - A.grp[i]) * S, nt = A.off[i + 1] - A.off[i];
+  const T *fc[S];
+  T *dst[S];
+  bool live[S]; // a fluid boundary cell (the halo of another is never read)
 #pragma unroll
-      for (int m = 0; m < NC; ++m) dst[(size_t)k * NC + m] = fc[(size_t)k * NC + m];
-    }
+  for (int j = 0; j < S; ++j) {
+    const long long t = min(t0 + j, nt - 1);
+    int ijk[3];
+    ijk[a] = (s > 0) ? A.n[a] - 1 : 0;
+    ijk[u] = (int)(t % A.n[u]);
+    ijk[v] = (int)(t / A.n[u]);
+    const long long c = ijk[0] + (long long)A.n[0] * (ijk[1] + (long long)A.n[1] * ijk[2]);
+    live[j] = t0 + j < nt && A.ctype[c] == IBDVM_CELL_FLUID;
+    fc[j] = A.f + (size_t)c * A.nvp * NC;
+    dst[j] = A.whalo + (size_t)(A.off[i] + t) * A.nvp * NC;
+    if (t0 + j < nt && !live[j])
+      for (int k = threadIdx.x; k < A.nvp * NC; k += blockDim.x) dst[j][k] = T(0);
+  }
+  const E *tab = A.tab + (size_t)i * A.nvp;
+  T so[S], eo[S];
+#pragma unroll
+  for (int j = 0; j < S; ++j) so[j] = eo[j] = T(0);
+  for (int k = threadIdx.x; k < A.nvp; k += blockDim.x) {
+    const E c = tab[k];
+    if (entering(c)) continue;
+#pragma unroll
+    for (int j = 0; j < S; ++j)
+      if (live[j]) {
+        T o[NC];
+        load_nc<T, NC>(fc[j] + (size_t)k * NC, o);
+        store_nc<T, NC>(dst[j] + (size_t)k * NC, o);
+        dot2(so[j], eo[j], c, o[0]);
+      }
+  }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int j = 0; j < S; ++j) {
+    double t = (double)so[j] + (double)eo[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) sh[j][wid] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x < S) {
+    double out = 0.0;
+    for (int w = 0; w < kDomainThreads / 32; ++w) out += sh[threadIdx.x][w];
+    const double rho_w = out / A.in[i]; // the table holds -M_w: (-rho_w) (-M_w)
+    split(rho_w, s_rho[0][threadIdx.x]);
+    split(A.halfT[i] * rho_w, s_rho[1][threadIdx.x]);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < A.nvp; k += blockDim.x) {
+    const E c = tab[k];
+    if (!entering(c)) continue;
+#pragma unroll
+    for (int j = 0; j < S; ++j)
+      if (live[j]) {
+        T o[NC];
+        o[0] = wall_value(s_rho[0][j], c);
+        if (NC == 2) o[NC - 1] = wall_value(s_rho[1][j], c); // B_w = T_w / 2 H_w
+        store_nc<T, NC>(dst[j] + (size_t)k * NC, o);
+      }
   }
 }
 
@@ -2087,20 +2146,24 @@ template <typename T, int D> cudaError_t domain_t(ibdvm_ctx *ctx) {
   DomainArgs<T> A{};
   A.f = static_cast<const T *>(ctx->f[ctx->cur]);
   A.ctype = ctx->ctype;
-  A.xiD = ctx->xiD;
-  A.wD = ctx->wD;
+  A.tab = static_cast<const typename WallEntry<T>::type *>(ctx->wall_tab);
   A.whalo = static_cast<T *>(ctx->whalo);
-  A.kst = ctx->kst;
   for (int i = 0; i < 7; ++i) A.off[i] = ctx->wall_off[i];
-  A.mask = ctx->wall_mask;
-  for (int a = 0; a < 3; ++a) A.n[a] = g.n[a];
-  A.nv = ctx->nv;
-  A.nvp = ctx->nvp;
+  long long walls = 0;
+  for (int i = 0; i < 6; ++i) walls += ((ctx->wall_mask >> i) & 1) ? A.off[i + 1] - A.off[i] : 0;
+  const int S = walls < kDomainFew ? 1 : kDomainSlots;
   for (int i = 0; i < 6; ++i) {
-    A.Tw[i] = ctx->wall_T[i];
-    for (int a = 0; a < 3; ++a) A.Uw[i][a] = ctx->wall_U[i][a];
+    const long long slots = ((ctx->wall_mask >> i) & 1) ? A.off[i + 1] - A.off[i] : 0;
+    A.grp[i + 1] = A.grp[i] + (int)((slots + S - 1) / S);
+    A.in[i] = ctx->wall_in[i];
+    A.halfT[i] = 0.5 * ctx->wall_T[i];
   }
-  domain_wall_kernel<T, D><<<(unsigned)ctx->wall_off[6], kDomainThreads, 0, ctx->stream>>>(A);
+  for (int a = 0; a < 3; ++a) A.n[a] = g.n[a];
+  A.nvp = ctx->nvp;
+  if (S == 1)
+    domain_wall_kernel<T, D, 1><<<(unsigned)A.grp[6], kDomainThreads, 0, ctx->stream>>>(A);
+  else
+    domain_wall_kernel<T, D, kDomainSlots><<<(unsigned)A.grp[6], kDomainThreads, 0, ctx->stream>>>(A);
   return cudaGetLastError();
 }
 
