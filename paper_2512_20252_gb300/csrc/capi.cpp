@@ -171,6 +171,9 @@ void free_all(ibdvm_ctx *ctx) {
   cfree_t(ctx->tree_lrec);
   cfree_t(ctx->tree_far);
   cfree_t(ctx->tree_sched);
+  cfree_t(ctx->plan64.grp);
+  cfree_t(ctx->plan64.nodes);
+  cfree_t(ctx->plan64.tab);
   cfree_t(ctx->partf);
   cfree_t(ctx->d_forces);
   cfree_t(ctx->d_step_forces);
@@ -713,6 +716,8 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
     int nchunk = static_cast<int>(std::min<long long>(kblocks, std::max<long long>(1, (4 * 152 + cell_blocks - 1) / cell_blocks)));
     ctx->kloop = (kblocks + nchunk - 1) / nchunk;
     ctx->nchunk = (kblocks + ctx->kloop - 1) / ctx->kloop;
+    const bool fp64_sweep = ctx->precision == IBDVM_FP64 && !tree;
+    if (fp64_sweep) ctx->nchunk = sweep64_nchunk(G);
     const int NW = G.dim + 2;
     const int NM = nmoments(G.dim);
     // memory check before allocating
@@ -767,6 +772,22 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
       ctx->oct_sign = dalloc<uint8_t>(ctx, sign.size(), "chunk signs");
       upload(ctx, ctx->oct_const, vconst, "upload velocity constants");
       upload(ctx, ctx->oct_sign, sign, "upload chunk signs");
+    }
+    if (fp64_sweep) {
+      std::vector<int> grp;
+      std::vector<double> nodes;
+      cudaError_t e = sweep64_prepare(ctx, grp, nodes);
+      if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        ctx->err = "device allocation of the equilibrium tables failed";
+        throw Fail{IBDVM_E_NOMEM};
+      }
+      check(ctx, e, "FP64 sweep set-up");
+      ctx->dev_bytes += ctx->plan64.tab_bytes;
+      ctx->plan64.grp = dalloc<int>(ctx, grp.size(), "velocity groups");
+      ctx->plan64.nodes = dalloc<double>(ctx, nodes.size(), "velocity nodes");
+      upload(ctx, ctx->plan64.grp, grp, "upload velocity groups");
+      upload(ctx, ctx->plan64.nodes, nodes, "upload velocity nodes");
     }
     // the TMA sweeps of FP32 cases
     if (!tma_off && (tma_sweep_applicable(ctx) || tma3_sweep_applicable(ctx))) {
@@ -1407,7 +1428,12 @@ size_t estimate_ctx_bytes(const ibdvm_grid_desc *grid, const ibdvm_vgrid_desc *v
   const int D = G.dim, NW = D + 2, NM = nmoments(D);
   size_t b = 2 * nc * nvp * G.ncomp * es;                               // f^n, f^{n+1}
   b += nc * (nvp / 64 + 1) * 4 * NM;                                     // FP32 moment partial sums
-  b += nc * (kMac * es + 2 * (NW + D) * 8 + (nvp / 64 + 1) * NM * 8 + 16); // per-cell state, FP64 sums
+  size_t chunks = nvp / 64 + 1;
+  if (gas->precision == IBDVM_FP64) { // the FP64 sweep's chunks and tables
+    chunks = std::max(chunks, static_cast<size_t>(sweep64_nchunk(G)));
+    b += sweep64_table_bytes(G);
+  }
+  b += nc * (kMac * es + 2 * (NW + D) * 8 + chunks * NM * 8 + 16); // per-cell state, FP64 sums
   // the ghost band: at most D n^(D-1) links for a body that fits the domain
   const double nl = D * std::pow(static_cast<double>(nc), (D - 1.0) / D);
   b += static_cast<size_t>(nl) * (nvp * (3 * G.ncomp * es + 8) + 256);

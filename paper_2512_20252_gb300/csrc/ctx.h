@@ -42,6 +42,22 @@ enum : int { kFlagNonFinite = 1, kFlagUnstable = 2, kFlagTimeout = 4 };
 
 struct ibdvm_batch; // batch.cpp
 
+namespace ibdvm {
+// cell flags (ctx->cmask): a cell that is not fluid
+constexpr unsigned kNotFluidCell = 64;
+
+// the FP64 sweep's work split and tables (sweep64.cu)
+struct Sweep64Plan {
+  int nbatch = 0, per = 0; // batches of velocity groups, per chunk of the moment sums
+  int rows = 0, slab = 0;  // rows of the last axis per block, and per launch
+  int nnode = 0;           // velocity nodes of all axes
+  int *grp = nullptr;      // the groups
+  double *nodes = nullptr; // [3][nnode]: component, dt |xi| / dx, width
+  double *tab = nullptr;   // per cell of a slab and axis node: the equilibrium's factors
+  size_t tab_bytes = 0;
+};
+} // namespace ibdvm
+
 struct ibdvm_ctx {
   ibdvm::Geom geom;
   cudaStream_t stream = nullptr;
@@ -77,6 +93,7 @@ struct ibdvm_ctx {
   uint8_t *ctype = nullptr;
   uint8_t *cmask = nullptr;  // per cell: ghost neighbour per face (bit 2a + (s > 0)), 64 = not fluid
   int *dslot = nullptr, *dlinks = nullptr;
+  ibdvm::Sweep64Plan plan64; // FP64 on a uniform grid (sweep64.cu)
   // TMA sweep of 2D FP32 cases (sweep_tma.cu)
   bool use_tma = false;
   float *partf = nullptr;    // FP32 moment partial sums [nchunk][9][ncell]
@@ -172,6 +189,14 @@ bool tma_sweep_applicable(const ibdvm_ctx *ctx);
 int tma_sweep_nchunk(const ibdvm_ctx *ctx);
 cudaError_t tma_sweep_prepare(ibdvm_ctx *ctx);
 cudaError_t tma_sweep_launch(ibdvm_ctx *ctx);
+// FP64 sweep of uniform grids (sweep64.cu): the chunks of its moment sums, the
+// bytes of its tables (fewer when memory is short), its set-up (groups and
+// axis nodes for the caller to upload) and one step's launches
+int sweep64_nchunk(const Geom &G);
+size_t sweep64_table_bytes(const Geom &G);
+cudaError_t sweep64_prepare(ibdvm_ctx *ctx, std::vector<int> &grp, std::vector<double> &nodes);
+int sweep64_launches(const ibdvm_ctx *ctx);
+cudaError_t sweep64_launch(ibdvm_ctx *ctx);
 // The orthant layout of the velocities for the FP32 TMA sweeps (layout.cpp):
 // chunks whose components have one sign each (quadrants in 2D, octants in
 // 3D).  orthant_layout gives the stored position of every velocity of G

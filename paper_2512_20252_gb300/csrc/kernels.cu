@@ -2360,10 +2360,15 @@ cudaError_t launch_sweep(ibdvm_ctx *ctx) {
     const bool tma = std::is_same<T, float>::value && ctx->use_tma;
     {
       Timed tm(ctx, kKSweep);
-      ctx->kernel_launches[kKSweep] += 1;
-      e = ctx->tree ? tree_sweep_t<T, D>(ctx)
-          : tma     ? (D == 2 ? tma_sweep_launch(ctx) : tma3_sweep_launch(ctx))
-                    : sweep_t<T, D>(ctx, 1, 1);
+      if constexpr (std::is_same<T, double>::value) {
+        ctx->kernel_launches[kKSweep] += ctx->tree ? 1 : sweep64_launches(ctx);
+        e = ctx->tree ? tree_sweep_t<T, D>(ctx) : sweep64_launch(ctx);
+      } else {
+        ctx->kernel_launches[kKSweep] += 1;
+        e = ctx->tree ? tree_sweep_t<T, D>(ctx)
+            : tma     ? (D == 2 ? tma_sweep_launch(ctx) : tma3_sweep_launch(ctx))
+                      : sweep_t<T, D>(ctx, 1, 1);
+      }
     }
     if (e != cudaSuccess) return e;
     ctx->cur = 1 - ctx->cur;
