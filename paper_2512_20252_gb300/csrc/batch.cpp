@@ -174,12 +174,12 @@ void one_step(ibdvm_batch *b, int p) {
   {
     BTimed t(b, kKGhost);
     bcheck(b, group_ghost(b->gt, p, b->stream), "grouped ghost-band kernel");
-    b->kernel_launches[kKGhost] += b->gt.link_blocks ? 1 : 0;
+    b->kernel_launches[kKGhost] += (b->gt.slope_blocks ? 1 : 0) + (b->gt.ghost_blocks ? 1 : 0);
   }
   {
     BTimed t(b, kKForces);
     bcheck(b, group_forces(b->gt, p, b->stream), "grouped force kernels");
-    b->kernel_launches[kKForces] += (b->gt.link_blocks ? 1 : 0) + 1;
+    b->kernel_launches[kKForces] += b->gt.link_blocks ? 1 : 0;
   }
   {
     BTimed t(b, kKSweep);

@@ -12,6 +12,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "ctx.h"
@@ -127,14 +128,23 @@ std::vector<double> wall_table(const ibdvm_ctx *ctx, const ibdvm_domain_desc &d,
   return t;
 }
 
+// FP64 values in the storage type of the context
+void upload_typed(ibdvm_ctx *ctx, void *dst, const std::vector<double> &src, const char *what) {
+  if (ctx->precision == IBDVM_FP64)
+    upload(ctx, static_cast<double *>(dst), src, what);
+  else
+    upload(ctx, static_cast<float *>(dst), cast<float>(src), what);
+}
+
+// the ghost band's device tables, all in one allocation
+struct BodyTable {
+  void **p;
+  size_t bytes;
+};
+
 void free_body(ibdvm_ctx *ctx) {
-  void *ps[] = {ctx->dslot, ctx->dlinks, ctx->l_int, ctx->l_dbl, ctx->l_wg, ctx->g_int, ctx->s_int,
-                ctx->s_dbl, ctx->lval, ctx->fi_scr, ctx->fsp_scr, ctx->rhow, ctx->fpart, ctx->gw_unit};
-  for (void *p : ps)
-    if (p) cudaFree(p);
-  ctx->dslot = ctx->dlinks = ctx->l_int = ctx->g_int = ctx->s_int = nullptr;
-  ctx->l_dbl = ctx->l_wg = ctx->s_dbl = ctx->rhow = ctx->fpart = ctx->gw_unit = nullptr;
-  ctx->lval = ctx->fi_scr = ctx->fsp_scr = nullptr;
+  cfree(ctx->body_mem); // the tables' pointers are set again with the next body
+  ctx->nlink = 0;
 }
 
 void drop_graphs(ibdvm_ctx *ctx) {
@@ -256,8 +266,9 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
   // surface entries: neighbour codes and the vectors of the weights and slopes
   const int mode = (G.gas.flags & IBDVM_RHAT_GHOST_TO_FLUID) ? 2 : 1;
   const size_t ns = G.surf_cell.size();
-  std::vector<int> s_int(8 * ns, -2);
+  std::vector<int> e_int(ns), c_int;
   std::vector<double> s_dbl(8 * ns, 0.0);
+  std::unordered_map<int, int> cells; // surface cell (of GS) -> index into c_int
   auto ijk_of = [&](long long c, int *o) {
     o[0] = static_cast<int>(c % GS.n[0]);
     o[1] = static_cast<int>((c / GS.n[0]) % GS.n[1]);
@@ -270,24 +281,28 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
       const int j = GS.surf_cell[e];
       int ij[3];
       ijk_of(j, ij);
-      int *si = &s_int[8 * e];
       double *sd = &s_dbl[8 * e];
-      si[0] = cell_of(j);
-      for (int a = 0; a < 3; ++a)
-        for (int s = 0; s < 2; ++s) {
-          int code = -2;
-          if (a < D) {
-            int q[3] = {ij[0], ij[1], ij[2]};
-            q[a] += s ? 1 : -1;
-            if (q[a] < 0 || q[a] >= GS.n[a]) {
-              code = -1; // domain halo: freestream or a diffuse domain wall
-            } else {
-              long long nb = q[0] + GS.n[0] * (q[1] + static_cast<long long>(GS.n[1]) * q[2]);
-              if (GS.type[nb] == IBDVM_CELL_FLUID) code = cell_of(nb);
+      const auto it = cells.emplace(j, static_cast<int>(cells.size()));
+      e_int[e] = it.first->second;
+      if (it.second) {
+        c_int.push_back(cell_of(j));
+        for (int a = 0; a < 3; ++a)
+          for (int s = 0; s < 2; ++s) {
+            int code = -2;
+            if (a < D) {
+              int q[3] = {ij[0], ij[1], ij[2]};
+              q[a] += s ? 1 : -1;
+              if (q[a] < 0 || q[a] >= GS.n[a]) {
+                code = -1; // domain halo: freestream or a diffuse domain wall
+              } else {
+                long long nb = q[0] + GS.n[0] * (q[1] + static_cast<long long>(GS.n[1]) * q[2]);
+                if (GS.type[nb] == IBDVM_CELL_FLUID) code = cell_of(nb);
+              }
             }
+            c_int.push_back(code);
           }
-          si[1 + 2 * a + s] = code;
-        }
+        c_int.push_back(0);
+      }
       double rl = 0.0;
       for (int a = 0; a < D; ++a) {
         const int o = (mode == 2) ? (ij[a] - ig[a]) : (ig[a] - ij[a]);
@@ -298,6 +313,13 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
       for (int a = 0; a < D; ++a) sd[4 + a] = (ij[a] - ig[a]) * G.dx[a];
       sd[7] = 1.0 / sd[3];
     }
+  }
+  std::vector<int> g_int(4 * G.ghosts.size());
+  for (size_t gi = 0; gi < G.ghosts.size(); ++gi) {
+    g_int[4 * gi] = G.ghost_first[gi];
+    g_int[4 * gi + 1] = G.ghost_nlinks[gi];
+    g_int[4 * gi + 2] = G.surf_off[gi];
+    g_int[4 * gi + 3] = G.surf_off[gi + 1];
   }
   std::vector<uint8_t> ctype(G.type.begin(), G.type.end());
   // per-cell flags of the sweeps: a ghost across face (a, s) sets bit 2a + (s > 0)
@@ -319,47 +341,45 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
         if (G.type[nb] == IBDVM_CELL_GHOST) cmask[c] |= static_cast<uint8_t>(1u << (2 * a + s));
       }
   }
-  // allocate the new band first, so that a failure leaves the old one intact
-  ibdvm_ctx tmp;
-  tmp.stream = ctx->stream;
-  try {
-    tmp.dslot = dalloc<int>(&tmp, dslot.size(), "donor slots");
-    tmp.dlinks = dalloc<int>(&tmp, dlinks.size(), "donor links");
-    tmp.l_int = dalloc<int>(&tmp, l_int.size(), "link table");
-    tmp.l_dbl = dalloc<double>(&tmp, l_dbl.size(), "link coefficients");
-    tmp.l_wg = dalloc<double>(&tmp, l_wg.size(), "cut table");
-    tmp.s_int = dalloc<int>(&tmp, s_int.size(), "surface table");
-    tmp.s_dbl = dalloc<double>(&tmp, s_dbl.size(), "surface vectors");
-    const size_t band = nl * static_cast<size_t>(nvp) * ctx->ncomp * ctx->esize;
-    tmp.lval = dalloc<char>(&tmp, band, "ghost values");
-    tmp.fi_scr = dalloc<char>(&tmp, band, "incident scratch");
-    tmp.fsp_scr = dalloc<char>(&tmp, band, "shifted-point scratch");
-    tmp.rhow = dalloc<double>(&tmp, nl, "wall density");
-    tmp.fpart = dalloc<double>(&tmp, 4 * nl, "force partial sums");
-    tmp.gw_unit = dalloc<double>(&tmp, nvp, "wall Maxwellian");
-  } catch (const Fail &f) {
-    ctx->err = tmp.err;
-    free_body(&tmp);
-    throw;
-  }
+  // allocate the new band first, so that a failure leaves the old one intact;
+  // one allocation for all its tables (each cudaMalloc costs a fraction of a
+  // millisecond beside a large state)
+  const size_t band = nl * static_cast<size_t>(nvp) * ctx->ncomp * ctx->esize;
+  const size_t nlv = nl * static_cast<size_t>(nvp), nsc = c_int.size() / 8;
+  const BodyTable tables[] = {
+      {(void **)&ctx->dslot, dslot.size() * sizeof(int)},
+      {(void **)&ctx->dlinks, dlinks.size() * sizeof(int)},
+      {(void **)&ctx->l_int, l_int.size() * sizeof(int)},
+      {(void **)&ctx->l_dbl, l_dbl.size() * sizeof(double)},
+      {(void **)&ctx->l_wg, nlv * sizeof(double)},
+      {(void **)&ctx->l_cn, nlv * sizeof(double)},
+      {&ctx->l_al, nlv * ctx->esize},
+      {(void **)&ctx->g_int, g_int.size() * sizeof(int)},
+      {(void **)&ctx->e_int, e_int.size() * sizeof(int)},
+      {(void **)&ctx->c_int, c_int.size() * sizeof(int)},
+      {&ctx->sig, nsc * D * nvp * ctx->ncomp * ctx->esize},
+      {&ctx->s_T, s_dbl.size() * ctx->esize},
+      {&ctx->lval, band},
+      {&ctx->fi_scr, band},
+      {&ctx->fsp_scr, band},
+      {(void **)&ctx->rhow, nl * sizeof(double)},
+      {(void **)&ctx->fpart, kForceParts * nl * sizeof(double)},
+      {(void **)&ctx->fcount, sizeof(int)},
+      {(void **)&ctx->gw_unit, nvp * sizeof(double)},
+      {&ctx->gw_T, nvp * ctx->esize},
+  };
+  size_t total = 0;
+  for (const BodyTable &t : tables) total += (t.bytes + 255) & ~size_t(255);
+  char *mem = dalloc<char>(ctx, total, "ghost band");
   free_body(ctx);
-  ctx->dev_bytes += tmp.dev_bytes;
-  ctx->dslot = tmp.dslot;
-  ctx->dlinks = tmp.dlinks;
-  ctx->l_int = tmp.l_int;
-  ctx->l_dbl = tmp.l_dbl;
-  ctx->l_wg = tmp.l_wg;
-  ctx->s_int = tmp.s_int;
-  ctx->s_dbl = tmp.s_dbl;
-  ctx->lval = tmp.lval;
-  ctx->fi_scr = tmp.fi_scr;
-  ctx->fsp_scr = tmp.fsp_scr;
-  ctx->rhow = tmp.rhow;
-  ctx->fpart = tmp.fpart;
-  ctx->gw_unit = tmp.gw_unit;
-  tmp.dslot = tmp.dlinks = tmp.l_int = tmp.s_int = nullptr;
-  tmp.l_dbl = tmp.l_wg = tmp.s_dbl = tmp.rhow = tmp.fpart = tmp.gw_unit = nullptr;
-  tmp.lval = tmp.fi_scr = tmp.fsp_scr = nullptr;
+  ctx->dev_bytes -= ctx->body_bytes;
+  ctx->body_mem = mem;
+  ctx->body_bytes = total;
+  for (const BodyTable &t : tables) {
+    *t.p = mem;
+    mem += (t.bytes + 255) & ~size_t(255);
+  }
+  ctx->nsc = static_cast<int>(nsc);
   ctx->nlink = static_cast<int>(nl);
   ctx->nghost = static_cast<int>(G.ghosts.size());
   ctx->nsurf = static_cast<int>(ns);
@@ -368,8 +388,11 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
   upload(ctx, ctx->l_int, l_int, "upload link table");
   upload(ctx, ctx->l_dbl, l_dbl, "upload link coefficients");
   upload(ctx, ctx->l_wg, l_wg, "upload cut table");
-  upload(ctx, ctx->s_int, s_int, "upload surface table");
-  upload(ctx, ctx->s_dbl, s_dbl, "upload surface vectors");
+  upload(ctx, ctx->g_int, g_int, "upload ghost table");
+  upload(ctx, ctx->e_int, e_int, "upload surface entries");
+  upload(ctx, ctx->c_int, c_int, "upload surface cells");
+  upload_typed(ctx, ctx->s_T, s_dbl, "upload surface vectors");
+  check(ctx, cudaMemsetAsync(ctx->fcount, 0, sizeof(int), ctx->stream), "clear force counter");
   {
     // unit-density wall Maxwellian per velocity (Eq. boundary maxwell; the 2D
     // reduced H_w of Sec. 4): depends on the wall only, so tabulated once
@@ -385,11 +408,12 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
       gw[ctx->kst_h[k]] = norm * std::exp(-c2 / Tw);
     }
     upload(ctx, ctx->gw_unit, gw, "upload wall Maxwellian");
+    upload_typed(ctx, ctx->gw_T, gw, "upload wall Maxwellian");
   }
+  check(ctx, launch_ghost_tables(ctx), "ghost tables kernel");
   upload(ctx, ctx->ctype, ctype, "upload cell classes");
   upload(ctx, ctx->cmask, cmask, "upload cell flags");
   if (nl) {
-    const size_t band = nl * static_cast<size_t>(nvp) * ctx->ncomp * ctx->esize;
     check(ctx, cudaMemsetAsync(ctx->lval, 0, band, ctx->stream), "clear ghost values");
     check(ctx, cudaMemsetAsync(ctx->fi_scr, 0, band, ctx->stream), "clear scratch");
     check(ctx, cudaMemsetAsync(ctx->fsp_scr, 0, band, ctx->stream), "clear scratch");
@@ -817,11 +841,18 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
     ctx->xiD = dalloc<double>(ctx, xi3.size(), "velocities");
     upload(ctx, ctx->xiD, xi3, "upload velocities");
     {
-      // the weights, followed by their reciprocals (zero at padding positions)
-      std::vector<double> w2(2 * w.size(), 0.0);
-      for (size_t k = 0; k < w.size(); ++k) {
+      // the weights, followed by their reciprocals, w xi per axis and |xi|^2 / 2
+      // (zero at padding positions)
+      const size_t np = w.size();
+      std::vector<double> w2(6 * np, 0.0);
+      for (size_t k = 0; k < np; ++k) {
         w2[k] = w[k];
-        w2[w.size() + k] = (w[k] > 0.0) ? 1.0 / w[k] : 0.0;
+        w2[np + k] = (w[k] > 0.0) ? 1.0 / w[k] : 0.0;
+        for (int a = 0; a < 3; ++a) {
+          const double x = xi3[a * np + k];
+          w2[(2 + a) * np + k] = w[k] * x;
+          w2[5 * np + k] += 0.5 * x * x;
+        }
       }
       ctx->wD = dalloc<double>(ctx, w2.size(), "weights");
       upload(ctx, ctx->wD, w2, "upload weights");
@@ -1436,7 +1467,7 @@ size_t estimate_ctx_bytes(const ibdvm_grid_desc *grid, const ibdvm_vgrid_desc *v
   b += nc * (kMac * es + 2 * (NW + D) * 8 + chunks * NM * 8 + 16); // per-cell state, FP64 sums
   // the ghost band: at most D n^(D-1) links for a body that fits the domain
   const double nl = D * std::pow(static_cast<double>(nc), (D - 1.0) / D);
-  b += static_cast<size_t>(nl) * (nvp * (3 * G.ncomp * es + 8) + 256);
+  b += static_cast<size_t>(nl) * (nvp * ((3 + 3 * D / 2.0) * G.ncomp * es + 16 + es) + 512);
   return b + nvp * 64 + (1u << 20);
 }
 

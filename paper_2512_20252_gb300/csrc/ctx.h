@@ -32,6 +32,9 @@ enum KernelClass { kKGhost = 0, kKSweep = 1, kKMoments = 2, kKForces = 3, kKOthe
 // columns of the wall-point quantities (ibdvm_wall)
 constexpr int kWallCols = 12;
 
+// force partial sums of a link (4 doubles for each of its blocks)
+constexpr int kForceParts = 16;
+
 // cell ranges of a pipelined host upload of the state (ibdvm_set_f_native)
 constexpr int kUploadParts = 8;
 
@@ -78,7 +81,8 @@ struct ibdvm_ctx {
   int *d_flags = nullptr;
   // velocity tables, indexed by the stored position of a velocity
   void *xiT = nullptr, *wT = nullptr, *finf = nullptr;
-  double *xiD = nullptr, *wD = nullptr; // wD: [2][nvp], the weights then their reciprocals (0 at padding)
+  // wD: [6][nvp], the weights, their reciprocals (0 at padding), w xi per axis, |xi|^2 / 2
+  double *xiD = nullptr, *wD = nullptr;
   // stored position of every velocity in its natural order (x index fastest):
   // the identity, or, for the orthant layout of the FP32 TMA sweeps,
   // velocities grouped by the signs of their components with each group
@@ -100,20 +104,29 @@ struct ibdvm_ctx {
   int tma_nchunk = 0;
   alignas(64) unsigned char tmap[2][128];
   alignas(64) unsigned char tmap3[2][3][128]; // 3D: tile, x halo strip, y halo strip per buffer
-  // ghost band
+  // ghost band (its tables lie in one allocation)
+  void *body_mem = nullptr;
+  size_t body_bytes = 0;
   int nlink = 0, nghost = 0, nsurf = 0;
   int *l_int = nullptr;      // [nlink][8]
   double *l_dbl = nullptr;   // [nlink][8]
   double *l_wg = nullptr;    // [nlink][nvp]
-  int *g_int = nullptr;      // [nghost][4]
-  int *s_int = nullptr;      // [nsurf][8]
-  double *s_dbl = nullptr;   // [nsurf][8]
+  double *l_cn = nullptr;    // [nlink][nvp] incident mass flux per unit f (ghost_tables_kernel)
+  void *l_al = nullptr;      // [nlink][nvp] incident share of a velocity's box
+  int *g_int = nullptr;      // [nghost][4]: first link, links, first and last + 1 surface entry
+  int *e_int = nullptr;      // [nsurf] surface cell of each entry
+  int *c_int = nullptr;      // [nsc][8]: cell, codes of its face neighbours
+  int nsc = 0;               // distinct surface cells
+  void *sig = nullptr;       // [nsc][dim][nvp][ncomp] their pre-ghost slopes
+  void *s_T = nullptr;       // [nsurf][8] in the storage type
   void *lval = nullptr;      // [nlink][nvp][ncomp] ghost values f*_gc
   void *fi_scr = nullptr;    // [nlink][nvp][ncomp] incident distribution at the wall
   void *fsp_scr = nullptr;   // [nlink][nvp][ncomp] shifted-point value
   double *rhow = nullptr;    // [nlink]
-  double *fpart = nullptr;   // [nlink][4] force partial sums
+  double *fpart = nullptr;   // force partial sums (kForceParts per link)
+  int *fcount = nullptr;     // blocks of a force launch done (zero between launches)
   double *gw_unit = nullptr; // [nvp] unit-density wall Maxwellian H_w / g_w of the body's wall
+  void *gw_T = nullptr;      // the same in the storage type
   double *d_forces = nullptr; // [4]
   double *d_step_forces = nullptr; // [4] forces of the fluxes the last step applied
   // kernel timing (CUDA events around each launch class, when enabled)
@@ -184,6 +197,8 @@ cudaError_t launch_wall(ibdvm_ctx *ctx, const double *fstar, double *out);
 cudaError_t launch_ghost_band(ibdvm_ctx *ctx, double *dbg_fstarw);
 cudaError_t launch_sweep(ibdvm_ctx *ctx);
 cudaError_t launch_forces(ibdvm_ctx *ctx, double *dst);
+// the ghost band's tables of the geometry and the wall (after a body is uploaded)
+cudaError_t launch_ghost_tables(ibdvm_ctx *ctx);
 // TMA sweep (sweep_tma.cu)
 bool tma_sweep_applicable(const ibdvm_ctx *ctx);
 int tma_sweep_nchunk(const ibdvm_ctx *ctx);
@@ -247,8 +262,10 @@ cudaError_t tma3_sweep_launch(ibdvm_ctx *ctx);
 struct GroupTables {
   int dim = 2, ncase = 0;
   void *ghost = nullptr, *force = nullptr, *fin = nullptr; // [ncase][2] argument blocks
-  int *link_start = nullptr, *fin_start = nullptr;         // [ncase + 1] block prefix sums
-  int link_blocks = 0, fin_blocks = 0;
+  // [ncase + 1] prefix sums: links, ghosts, blocks of the slope and finalize kernels
+  int *link_start = nullptr, *ghost_start = nullptr, *slope_start = nullptr, *fin_start = nullptr;
+  int link_blocks = 0, ghost_blocks = 0, slope_blocks = 0, fin_blocks = 0;
+  int split = 1; // blocks per ghost's cluster
 };
 cudaError_t group_build(const std::vector<ibdvm_ctx *> &cases, const std::vector<int> &nchunk, double *res,
                         int *flags, double *forces, GroupTables &t, cudaStream_t s);

@@ -20,6 +20,7 @@
 // Storage type T is double (FP64 path) or float (mixed path: FP32 f, FP32
 // transport and relaxation with compensated FP32 moment sums; FP64 wall
 // balance, forces and residual).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
@@ -38,16 +39,28 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr int kThreadsPerCell = 64; // threads over velocities for one cell
 constexpr int kCellsPerBlock = 4;   // cells of one sweep block
 constexpr int kBlock = kThreadsPerCell * kCellsPerBlock;
-constexpr int kGhostThreads = 512; // threads over the velocities of one link
-// The ghost band's tiling: U velocities a thread takes at a time, and blocks
-// of 512 threads per SM.  FP32 storage: two velocities at a time, two blocks
-// per SM (64 registers); FP64 storage and the grouped launches of a batch
-// (their arguments come from shared memory) need more registers: one block.
-template <typename T, bool GROUPED> struct GhostTiling {
-  static constexpr bool two = std::is_same<T, float>::value && !GROUPED;
-  static constexpr int U = 2;
-  static constexpr int blocks = two ? 2 : 1;
-};
+// The ghost band: a cluster of up to kGhostSplit blocks per ghost cell shares its
+// velocities and adds the wall-density sums through distributed shared memory,
+// so that a body of few ghosts still spreads over the chip.  What bounds it is
+// the latency of the gathers (FP64 storage: the FP64 pipe's).  Per step, both
+// kernels: 64^3 sphere (144 ghosts, 312 links, 20^3 velocities) 221 us, where one
+// block of 512 threads per link, two rounds of them, had taken 867; octree sphere
+// (672 links) 398 us (1487); 24^3 sphere in FP64 124 us (791).  Threads per block, and the
+// velocities a block of the slope kernel takes.
+constexpr int kGhostSplit = 8;
+constexpr int kGhostThreads = 128;
+constexpr int kSlopeVel = 4 * kGhostThreads;
+// blocks per cluster: as many as keep a velocity for every thread
+inline int ghost_split(int nvp) {
+  int s = kGhostSplit;
+  while (s > 1 && s * kGhostThreads > nvp) s /= 2;
+  return s;
+}
+// The surface force: kForceSplit blocks of kForceThreads per link; the last block
+// of a launch to finish adds their sums in a fixed order (one block per link and
+// a kernel for the total: 174 us on the 64^3 sphere, now 58; 27 us on 24 links, now 12)
+constexpr int kForceSplit = 4;
+constexpr int kForceThreads = 128;
 
 template <int D> struct Dims {
   static constexpr int NC = (D == 2) ? 2 : 1;   // components: (h, b) or f
@@ -210,6 +223,22 @@ __device__ __forceinline__ void seen(const SweepArgs<T> &A, long long c, const i
   } else {
     load_nc<T, NC>(A.f + ((size_t)nb * A.nvp + k) * NC, out);
   }
+}
+
+// the row [nvp][NC] of those values
+template <typename T, int NC>
+__device__ __forceinline__ const T *seen_row(const SweepArgs<T> &A, long long c, const int *ijk, int a, int s) {
+  const int q = ijk[a] + s, i = 2 * a + (s > 0);
+  if (q < 0 || q >= A.n[a]) {
+    if (!((A.H.mask >> i) & 1)) return A.finf;
+    return A.H.whalo + (size_t)(A.H.off[i] + face_slot(A.n, ijk, a)) * A.nvp * NC;
+  }
+  const long long stride = (a == 0) ? 1LL : (a == 1 ? (long long)A.n[0] : (long long)A.n[0] * A.n[1]);
+  const long long nb = c + s * stride;
+  if (A.ctype[nb] != IBDVM_CELL_GHOST) return A.f + (size_t)nb * A.nvp * NC;
+  const int slot = A.dslot[c];
+  const int l = (slot >= 0) ? A.dlinks[slot * 6 + i] : -1;
+  return (l >= 0) ? A.lval + (size_t)l * A.nvp * NC : A.finf;
 }
 
 template <typename T> __device__ __forceinline__ T shfl_down(T v, int o) {
@@ -1207,11 +1236,17 @@ template <typename T> struct GhostArgs {
   const double *__restrict__ rwD; // [nvp]: 1 / w (0 at padding positions)
   const T *__restrict__ xiT;
   const int *__restrict__ l_int;  // [nlink][8]: gidx, donor, aux, axis, side, ghost, s0, s1
-  const double *__restrict__ l_dbl; // [nlink][8]: c_sp, c_iw, c_gc, n0, n1, n2, S, -
-  const double *__restrict__ l_wg;  // [nlink][nvp]
-  const int *__restrict__ s_int;    // [nsurf][8]: cell, codes of the 6 face neighbours
-  const double *__restrict__ s_dbl; // [nsurf][8]: r (weights), |r|, x_j - x_g, 1 / |r|
+  const double *__restrict__ l_dbl; // [nlink][8]: c_sp, c_iw, c_gc, n0, n1, n2, S, sum of ws xn G_w
+  const double *__restrict__ l_wg;  // [nlink][nvp] incident-side measures
+  const double *__restrict__ l_cn;  // [nlink][nvp]: wg xn, the incident mass flux per unit f
+  const T *__restrict__ l_al;       // [nlink][nvp]: wg / w, the incident share of a velocity's box
+  const int *__restrict__ g_int;    // [nghost][4]: first link, links, first and last + 1 surface entry
+  const int *__restrict__ e_int;    // [nsurf]: the surface cell of an entry (index into c_int)
+  const int *__restrict__ c_int;    // [nsc][8]: surface cell, codes of its 6 face neighbours
+  const T *__restrict__ s_T;        // [nsurf][8]: r (weights), |r|, x_j - x_g, 1 / |r|
+  T *__restrict__ sig;              // [nsc][D][nvp][NC]: pre-ghost slopes of the surface cells
   const double *__restrict__ gwu;   // [nvp] unit-density wall Maxwellian
+  const T *__restrict__ gwT;        // the same in the storage type
   const int *__restrict__ kst;      // [nv] stored position of each velocity (natural order)
   T *__restrict__ lval;
   T *__restrict__ fi;
@@ -1219,6 +1254,7 @@ template <typename T> struct GhostArgs {
   double *__restrict__ rhow;
   double *__restrict__ dbg_fstar; // optional [nlink][nvp][NC] (FP64)
   int nv, nvp;
+  int split; // blocks that share a ghost's velocities (a batch's clusters may have more: they add zeros)
   int nvx[3];
   double vx0[3], vh[3]; // first node and node spacing per axis (mirror interpolation)
   double dx[3];
@@ -1247,29 +1283,56 @@ template <int NT> __device__ __forceinline__ double block_sum(double v, double *
   return sh[NT / 32];
 }
 
-// pre-ghost slope of surface cell j along axis a: van Leer with two fluid or
-// halo neighbours, one-sided with one, zero with none
-template <typename T, int NC>
-__device__ __forceinline__ T preghost_slope(const GhostArgs<T> &G, int code_m, int code_p, T fj,
-                                            int k, int m, T rh, int jc, int a) {
-  const bool hm = code_m != -2, hp = code_p != -2;
-  T fm = T(0), fp = T(0);
+// Pre-ghost slopes of surface cell jc along every axis, velocity k: van Leer with
+// two fluid or halo neighbours, one-sided with one, zero with none.  A surface
+// cell serves several ghosts (64^3 sphere: 416 cells for 1632 entries of 144
+// ghosts, and 3816 when every link forms them for itself), so its slopes are
+// formed once per step, by a kernel of their own.
+template <typename T, int D> __device__ __forceinline__ void surface_slopes_body(const GhostArgs<T> &G, const int blk) {
+  constexpr int NC = Dims<D>::NC;
+  const int nch = (G.nvp + kSlopeVel - 1) / kSlopeVel;
+  const int j = blk / nch, k0 = (blk % nch) * kSlopeVel + threadIdx.x;
+  const int *ci = G.c_int + 8 * j;
+  const int jc = ci[0];
   int ijk[3] = {0, 0, 0};
-  if (code_m == -1 || code_p == -1) { // a domain halo neighbour
+  bool halo = false;
+  for (int c = 0; c < 2 * D; ++c) halo = halo || ci[1 + c] == -1;
+  if (halo) { // a domain halo neighbour
     ijk[0] = jc % G.n[0];
     ijk[1] = (jc / G.n[0]) % G.n[1];
     ijk[2] = jc / (G.n[0] * G.n[1]);
   }
-  if (hm)
-    fm = (code_m >= 0) ? G.f[((size_t)code_m * G.nvp + k) * NC + m]
-                       : halo_value(G.H, G.finf, G.n, ijk, a, -1, G.nvp, NC, k, m);
-  if (hp)
-    fp = (code_p >= 0) ? G.f[((size_t)code_p * G.nvp + k) * NC + m]
-                       : halo_value(G.H, G.finf, G.n, ijk, a, +1, G.nvp, NC, k, m);
-  if (hm && hp) return vanleer((fj - fm) * rh, (fp - fj) * rh);
-  if (hm) return (fj - fm) * rh;
-  if (hp) return (fp - fj) * rh;
-  return T(0);
+  T rdx[D];
+  for (int a = 0; a < D; ++a) rdx[a] = (T)(1.0 / G.dx[a]);
+#pragma unroll
+  for (int u = 0; u < kSlopeVel / kGhostThreads; ++u) {
+    const int k = k0 + u * kGhostThreads;
+    if (k >= G.nvp) break;
+    T fj[NC];
+    load_nc<T, NC>(G.f + ((size_t)jc * G.nvp + k) * NC, fj);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      const int cm = ci[1 + 2 * a], cp = ci[2 + 2 * a];
+      T fm[NC], fp[NC], o[NC];
+#pragma unroll
+      for (int m = 0; m < NC; ++m) fm[m] = fp[m] = fj[m];
+      if (cm >= 0) load_nc<T, NC>(G.f + ((size_t)cm * G.nvp + k) * NC, fm);
+      if (cp >= 0) load_nc<T, NC>(G.f + ((size_t)cp * G.nvp + k) * NC, fp);
+#pragma unroll
+      for (int m = 0; m < NC; ++m) {
+        if (cm == -1) fm[m] = halo_value(G.H, G.finf, G.n, ijk, a, -1, G.nvp, NC, k, m);
+        if (cp == -1) fp[m] = halo_value(G.H, G.finf, G.n, ijk, a, +1, G.nvp, NC, k, m);
+        const T dm = (fj[m] - fm[m]) * rdx[a], dp = (fp[m] - fj[m]) * rdx[a];
+        o[m] = (cm != -2 && cp != -2) ? vanleer(dm, dp) : (cm != -2) ? dm : (cp != -2) ? dp : T(0);
+      }
+      store_nc<T, NC>(G.sig + (((size_t)j * D + a) * G.nvp + k) * NC, o);
+    }
+  }
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kGhostThreads) surface_slopes_kernel(const __grid_constant__ GhostArgs<T> G) {
+  surface_slopes_body<T, D>(G, blockIdx.x);
 }
 
 // the node interval of the velocity grid holding coordinate x along axis a:
@@ -1307,247 +1370,310 @@ __device__ __forceinline__ bool mirror_bracket(const GhostArgs<T> &G, int a, dou
   return !(x < xl || x > xh);
 }
 
-// The ghost band of link l, one block: every thread takes U velocities at a
-// time (strided by the block), so that U independent chains of loads are in
-// flight per thread and the link's surface-cell entries are read once per U
-// velocities.
-template <typename T, int D, int U>
-__device__ __forceinline__ void ghost_band_body(const GhostArgs<T> &G, const int l) {
+// Sums of v[q], q < n, over the cluster's blocks in a fixed order, in every
+// thread; sh and slot: shared arrays, slot used by no other call of the kernel.
+template <int NQ>
+__device__ __forceinline__ void cluster_sums(double (&v)[NQ], int n, double (*sh)[NQ], double *slot) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q)
+    if (q < n) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+      if (lane == 0) sh[wid][q] = v[q];
+    }
+  __syncthreads();
+  if (threadIdx.x < n) {
+    double s = 0.0;
+    for (int w = 0; w < kGhostThreads / 32; ++w) s += sh[w][threadIdx.x];
+    slot[threadIdx.x] = s;
+  }
+  cl.sync();
+#pragma unroll
+  for (int q = 0; q < NQ; ++q)
+    if (q < n) {
+      double t = 0.0;
+      for (unsigned r = 0; r < cl.num_blocks(); ++r) t += *cl.map_shared_rank(slot + q, r);
+      v[q] = t;
+    }
+}
+
+// f^i at the mirrored velocity of stored position k by multilinear interpolation
+// (C13; zero outside the velocity grid): the specular part of link l
+template <typename T, int D>
+__device__ __forceinline__ void mirrored(const GhostArgs<T> &G, const int l, const int k, const double *nw, double &xn,
+                                         double *v) {
   constexpr int NC = Dims<D>::NC;
-  __shared__ double sh[kGhostThreads / 32 + 1];
-  const int *li = G.l_int + 8 * l;
-  const double *ld = G.l_dbl + 8 * l;
-  const int donor = li[1], aux = li[2], s0 = li[6], s1 = li[7];
-  const int ns = s1 - s0;
-  const double c_sp = ld[0], c_iw = ld[1], c_gc = ld[2];
-  const double nw[3] = {ld[3], ld[4], ld[5]};
+  xn = 0.0;
+  for (int a = 0; a < D; ++a) xn += G.xiD[a * G.nvp + k] * nw[a];
+  bool inside = true;
+  int i0[3] = {0, 0, 0};
+  double t[3] = {0, 0, 0};
+  for (int a = 0; a < D; ++a)
+    if (!mirror_bracket(G, a, G.xiD[a * G.nvp + k] - 2.0 * xn * nw[a], i0[a], t[a])) inside = false;
+#pragma unroll
+  for (int m = 0; m < NC; ++m) v[m] = 0.0;
+  if (!inside) return;
+  for (int corner = 0; corner < (1 << D); ++corner) {
+    double wt = 1.0;
+    int id[3] = {0, 0, 0};
+    for (int a = 0; a < D; ++a) {
+      const int b = (corner >> a) & 1;
+      id[a] = i0[a] + b;
+      wt *= b ? t[a] : 1.0 - t[a];
+    }
+    const int kk = G.kst[id[0] + G.nvx[0] * (id[1] + G.nvx[1] * id[2])];
+#pragma unroll
+    for (int m = 0; m < NC; ++m) v[m] += wt * (double)G.fi[((size_t)l * G.nvp + kk) * NC + m];
+  }
+}
+
+// The ghost band of ghost cell g (all its links) by a cluster of blocks, each
+// taking a range of the stored velocity positions (padding positions hold zero
+// f, weight and flux and get a zero ghost value): f_gc, which the links share,
+// then per link the shifted point, the incident distribution and, after the
+// cluster's sum for the wall density, the wall distribution and ghost value.
+template <typename T, int D> __device__ __forceinline__ void ghost_band_body(const GhostArgs<T> &G, const int g) {
+  constexpr int NC = Dims<D>::NC;
+  constexpr int NQ = 2 * D;                   // links of a ghost at most
+  constexpr int NE = (D == 2) ? 8 : 26;       // surface cells of a ghost at most
+  constexpr int U = (sizeof(T) == 4 && D == 3) ? 4 : 2; // velocities of a thread at a time
+  __shared__ double sh[kGhostThreads / 32][NQ];
+  __shared__ double s_sum[2][NQ]; // this block's shares of the sums N and S
+  // the ghost's entries and links: read once per block, then from shared memory
+  // by every velocity (their loads had been most of the instructions)
+  __shared__ __align__(16) T e_s[NE][8];
+  __shared__ const T *e_f[NE], *e_sig[NE];
+  __shared__ T q_c[NQ][2];            // c_sp, c_iw
+  __shared__ const T *q_d[NQ], *q_a[NQ]; // rows of the donor and the auxiliary cell (null: none)
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = cl.block_rank();
+  const int per = ((G.nvp + G.split - 1) / G.split + 31) & ~31; // positions of a block
+  const int k0 = min(G.nvp, rank * per), k1 = min(G.nvp, k0 + per);
+  const int *gi = G.g_int + 4 * g;
+  const int l0 = gi[0], nq = gi[1], s0 = gi[2], ns = gi[3] - s0;
   const double alpha = G.accom;
-  const double *wgl = G.l_wg + (size_t)l * G.nvp;
-  // per-link constants in the storage type, converted once (FP64 divisions
-  // and conversions run on GB300's narrow FP64 pipe)
-  T rdx[3];
-  for (int a = 0; a < 3; ++a) rdx[a] = (a < D) ? (T)(1.0 / G.dx[a]) : T(0);
-  const T csp = (T)c_sp, ciw = (T)c_iw, wfall = T(1) / T(ns > 0 ? ns : 1);
-  double Nsum = 0.0, Dsum = 0.0;
-  for (int iv0 = threadIdx.x; iv0 < G.nv; iv0 += U * blockDim.x) {
+  for (int i = threadIdx.x; i < ns * 8; i += kGhostThreads) e_s[i >> 3][i & 7] = G.s_T[8 * (size_t)s0 + i];
+  if (threadIdx.x < ns) {
+    const int c = G.e_int[s0 + threadIdx.x];
+    e_f[threadIdx.x] = G.f + (size_t)G.c_int[8 * c] * G.nvp * NC;
+    e_sig[threadIdx.x] = G.sig + (size_t)c * D * G.nvp * NC;
+  }
+  if (threadIdx.x >= 64 && threadIdx.x < 64 + nq) {
+    const int q = threadIdx.x - 64, l = l0 + q, aux = G.l_int[8 * l + 2];
+    q_c[q][0] = (T)G.l_dbl[8 * l];
+    q_c[q][1] = (T)G.l_dbl[8 * l + 1];
+    q_d[q] = G.f + (size_t)G.l_int[8 * l + 1] * G.nvp * NC;
+    q_a[q] = (aux >= 0) ? G.f + (size_t)aux * G.nvp * NC : nullptr;
+  }
+  __syncthreads();
+  const T wfall = T(1) / T(ns > 0 ? ns : 1);
+  double N[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) N[q] = 0.0;
+  for (int kb = k0 + threadIdx.x; kb < k1; kb += U * kGhostThreads) {
     int k[U];
-    bool ok[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int iv = iv0 + u * blockDim.x;
-      ok[u] = iv < G.nv;
-      k[u] = G.kst[ok[u] ? iv : iv0];
-    }
-    // upwind weights, Eq. upwind (FP64 for the exact-zero decision in the FP64 path)
-    T xiT[U][3];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      for (int a = 0; a < 3; ++a) xiT[u][a] = (a < D) ? G.xiT[a * G.nvp + k[u]] : T(0);
-    T wsum[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) wsum[u] = T(0);
-    for (int j = 0; j < (G.naive ? 0 : ns); ++j) {
-      const double *sd = G.s_dbl + 8 * (s0 + j);
-      T r[3];
-      for (int a = 0; a < 3; ++a) r[a] = (a < D) ? (T)sd[a] : T(0);
-      const T rinv = (T)sd[7];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        // xi.r without contraction: tangential velocities give an exact zero
-        T xr = T(0);
-        for (int a = 0; a < D; ++a) xr = add_rn(xr, mul_rn(xiT[u][a], r[a]));
-        const T dot = mul_rn(xr, rinv);
-        const T mx = dot > T(0) ? dot : T(0);
-        wsum[u] = add_rn(wsum[u], mul_rn(mx, mx));
-      }
-    }
+    for (int u = 0; u < U; ++u) k[u] = (kb + u * kGhostThreads < k1) ? kb + u * kGhostThreads : kb;
     T fgc[U][NC];
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int m = 0; m < NC; ++m) fgc[u][m] = T(0);
-    if (G.naive) { // the construction without upwind weighting, Sec. 3.3.4
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int m = 0; m < NC; ++m) {
-          const T fd = G.f[((size_t)donor * G.nvp + k[u]) * NC + m];
-          fgc[u][m] = (aux >= 0) ? T(2) * fd - G.f[((size_t)aux * G.nvp + k[u]) * NC + m] : fd;
-        }
-    }
-    for (int j = 0; j < (G.naive ? 0 : ns); ++j) {
-      const int *si = G.s_int + 8 * (s0 + j);
-      const double *sd = G.s_dbl + 8 * (s0 + j);
-      const int jc = si[0];
-      T r[3], dxg[3];
-      bool has[3];
-      for (int a = 0; a < 3; ++a) {
-        r[a] = (a < D) ? (T)sd[a] : T(0);
-        has[a] = (a < D) && sd[4 + a] != 0.0;
-        dxg[a] = (a < D) ? (T)sd[4 + a] : T(0);
-      }
-      const T rinv = (T)sd[7];
+    if (!G.naive) {
+      // upwind weights, Eq. upwind (FP64 for the exact-zero decision in the FP64 path)
+      T xi[U][D], wsum[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const bool fallback = G.plain_average || !(wsum[u] != T(0));
-        T wt;
-        if (fallback) {
-          wt = wfall;
-        } else {
-          T xr = T(0);
-          for (int a = 0; a < D; ++a) xr = add_rn(xr, mul_rn(xiT[u][a], r[a]));
-          const T dot = mul_rn(xr, rinv);
-          const T mx = dot > T(0) ? dot : T(0);
-          wt = mul_rn(mx, mx) / wsum[u];
-        }
+        wsum[u] = T(0);
 #pragma unroll
-        for (int m = 0; m < NC; ++m) {
-          const T fj = G.f[((size_t)jc * G.nvp + k[u]) * NC + m];
-          T v = fj; // f_j - sigma_j . (x_j - x_g)
-          for (int a = 0; a < D; ++a) {
-            if (has[a]) {
-              T sig = preghost_slope<T, NC>(G, si[1 + 2 * a], si[2 + 2 * a], fj, k[u], m, rdx[a], jc, a);
-              v -= sig * dxg[a];
+        for (int a = 0; a < D; ++a) xi[u][a] = G.xiT[a * G.nvp + k[u]];
+      }
+      // xi.r without contraction: tangential velocities give an exact zero
+      auto weight = [&](int u, const T *sd) {
+        T xr = T(0);
+#pragma unroll
+        for (int a = 0; a < D; ++a) xr = add_rn(xr, mul_rn(xi[u][a], sd[a]));
+        const T dot = mul_rn(xr, sd[7]);
+        const T mx = dot > T(0) ? dot : T(0);
+        return mul_rn(mx, mx);
+      };
+      for (int j = 0; j < ns; ++j)
+#pragma unroll
+        for (int u = 0; u < U; ++u) wsum[u] = add_rn(wsum[u], weight(u, e_s[j]));
+      bool fallback[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) fallback[u] = G.plain_average || !(wsum[u] != T(0));
+      for (int j = 0; j < ns; ++j) {
+        const T *sd = e_s[j], *fr = e_f[j], *sr = e_sig[j];
+        T v[U][NC]; // f_j - sigma_j . (x_j - x_g)
+#pragma unroll
+        for (int u = 0; u < U; ++u) load_nc<T, NC>(fr + (size_t)k[u] * NC, v[u]);
+#pragma unroll
+        for (int a = 0; a < D; ++a)
+          if (sd[4 + a] != T(0)) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              T sg[NC];
+              load_nc<T, NC>(sr + ((size_t)a * G.nvp + k[u]) * NC, sg);
+#pragma unroll
+              for (int m = 0; m < NC; ++m) v[u][m] -= sg[m] * sd[4 + a];
             }
           }
-          fgc[u][m] += wt * v;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const T wt = fallback[u] ? wfall : weight(u, sd) / wsum[u];
+#pragma unroll
+          for (int m = 0; m < NC; ++m) fgc[u][m] += wt * v[u][m];
         }
       }
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (!ok[u]) continue;
-      const int ku = k[u];
-      // shifted point (Eq. fsp) and incident distribution at the wall (Eq. fw)
-      T fiv0 = T(0);
+    for (int q = 0; q < NQ; ++q)
+      if (q < nq) {
+        const int l = l0 + q;
+        const T *dr = q_d[q], *ar = q_a[q];
+        const T csp = q_c[q][0], ciw = q_c[q][1];
 #pragma unroll
-      for (int m = 0; m < NC; ++m) {
-        const T fd = G.f[((size_t)donor * G.nvp + ku) * NC + m];
-        T sp = fd;
-        if (aux >= 0) sp = fd + csp * (G.f[((size_t)aux * G.nvp + ku) * NC + m] - fd);
-        const T fiv = sp + ciw * (fgc[u][m] - sp);
-        if (m == 0) fiv0 = fiv;
-        G.fsp[((size_t)l * G.nvp + ku) * NC + m] = sp;
-        G.fi[((size_t)l * G.nvp + ku) * NC + m] = fiv;
+        for (int u = 0; u < U; ++u) {
+          if (u > 0 && kb + u * kGhostThreads >= k1) continue;
+          // shifted point (Eq. fsp) and incident distribution at the wall (Eq. fw)
+          T fd[NC], fa[NC], sp[NC], fi[NC];
+          load_nc<T, NC>(dr + (size_t)k[u] * NC, fd);
+          if (ar) load_nc<T, NC>(ar + (size_t)k[u] * NC, fa);
+#pragma unroll
+          for (int m = 0; m < NC; ++m) {
+            sp[m] = ar ? fd[m] + csp * (fa[m] - fd[m]) : fd[m];
+            // without upwind weighting: 2 f_d - f_ac (Sec. 3.3.4)
+            const T gc = !G.naive ? fgc[u][m] : ar ? T(2) * fd[m] - fa[m] : fd[m];
+            fi[m] = sp[m] + ciw * (gc - sp[m]);
+          }
+          store_nc<T, NC>(G.fsp + ((size_t)l * G.nvp + k[u]) * NC, sp);
+          store_nc<T, NC>(G.fi + ((size_t)l * G.nvp + k[u]) * NC, fi);
+          // the incident mass flux of the zero-net-mass-flux balance with the
+          // cut-cell split (Eq. rhowc), FP64
+          N[q] += G.l_cn[(size_t)l * G.nvp + k[u]] * (double)fi[0];
+        }
       }
-      // zero-net-mass-flux balance with the cut-cell split (Eq. rhowc), FP64
-      double xn = 0.0;
-      for (int a = 0; a < D; ++a) xn += G.xiD[a * G.nvp + ku] * nw[a];
-      const double Gw = G.gwu[ku];
-      const double wg = wgl[ku], ws = G.wD[ku] - wg;
-      Nsum += wg * xn * (double)fiv0;
-      Dsum += ws * xn * Gw;
-    }
   }
-  __syncthreads(); // scratch writes of this block are visible to the block
-  const double N = block_sum<kGhostThreads>(Nsum, sh);
-  const double Dd = block_sum<kGhostThreads>(Dsum, sh);
-  double Ssum = 0.0;
+  // (the cluster barrier also makes the blocks' f^i visible to each other)
+  cluster_sums<NQ>(N, nq, sh, s_sum[0]);
+  double S[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) S[q] = 0.0;
   if (alpha < 1.0) {
-    // specular part: f^i at the mirrored velocity by multilinear interpolation
-    for (int iv = threadIdx.x; iv < G.nv; iv += blockDim.x) {
-      const int k = G.kst[iv];
-      double xn = 0.0;
-      for (int a = 0; a < D; ++a) xn += G.xiD[a * G.nvp + k] * nw[a];
-      double xm[3];
-      for (int a = 0; a < D; ++a) xm[a] = G.xiD[a * G.nvp + k] - 2.0 * xn * nw[a];
-      bool inside = true;
-      int i0[3] = {0, 0, 0};
-      double t[3] = {0, 0, 0};
-      for (int a = 0; a < D; ++a)
-        if (!mirror_bracket(G, a, xm[a], i0[a], t[a])) inside = false;
-      double v = 0.0;
-      if (inside)
-        for (int corner = 0; corner < (1 << D); ++corner) {
-          double wt = 1.0;
-          int id[3] = {0, 0, 0};
-          for (int a = 0; a < D; ++a) {
-            int b = (corner >> a) & 1;
-            id[a] = i0[a] + b;
-            wt *= b ? t[a] : 1.0 - t[a];
-          }
-          const int kk = G.kst[id[0] + G.nvx[0] * (id[1] + G.nvx[1] * id[2])];
-          v += wt * (double)G.fi[((size_t)l * G.nvp + kk) * NC];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+      if (q < nq) {
+        const int l = l0 + q;
+        const double nw[3] = {G.l_dbl[8 * l + 3], G.l_dbl[8 * l + 4], G.l_dbl[8 * l + 5]};
+        for (int k = k0 + threadIdx.x; k < k1; k += kGhostThreads) {
+          double xn, v[NC];
+          mirrored<T, D>(G, l, k, nw, xn, v);
+          S[q] += (G.wD[k] - G.l_wg[(size_t)l * G.nvp + k]) * xn * v[0];
         }
-      Ssum += (G.wD[k] - wgl[k]) * xn * v;
-    }
-  }
-  const double S = (alpha < 1.0) ? block_sum<kGhostThreads>(Ssum, sh) : 0.0;
-  const double rho_w = (alpha > 0.0) ? -(N + (1.0 - alpha) * S) / (alpha * Dd) : 0.0;
-  if (threadIdx.x == 0) G.rhow[l] = rho_w;
-  // wall distribution (Eqs. general bc, Maxwell BC, fwc) and ghost value (Eq. extrapolation 2)
-#pragma unroll U
-  for (int iv = threadIdx.x; iv < G.nv; iv += blockDim.x) {
-    const int k = G.kst[iv];
-    double xn = 0.0;
-    for (int a = 0; a < D; ++a) xn += G.xiD[a * G.nvp + k] * nw[a];
-    const double Gw = G.gwu[k];
-    double fsv[NC];
-#pragma unroll
-    for (int m = 0; m < NC; ++m) fsv[m] = 0.0;
-    if (alpha < 1.0) {
-      double xm[3];
-      for (int a = 0; a < D; ++a) xm[a] = G.xiD[a * G.nvp + k] - 2.0 * xn * nw[a];
-      bool inside = true;
-      int i0[3] = {0, 0, 0};
-      double t[3] = {0, 0, 0};
-      for (int a = 0; a < D; ++a)
-        if (!mirror_bracket(G, a, xm[a], i0[a], t[a])) inside = false;
-      if (inside)
-        for (int corner = 0; corner < (1 << D); ++corner) {
-          double wt = 1.0;
-          int id[3] = {0, 0, 0};
-          for (int a = 0; a < D; ++a) {
-            int b = (corner >> a) & 1;
-            id[a] = i0[a] + b;
-            wt *= b ? t[a] : 1.0 - t[a];
-          }
-          const int kk = G.kst[id[0] + G.nvx[0] * (id[1] + G.nvx[1] * id[2])];
-#pragma unroll
-          for (int m = 0; m < NC; ++m) fsv[m] += wt * (double)G.fi[((size_t)l * G.nvp + kk) * NC + m];
-        }
-    }
-    const double wk = G.wD[k], wg = wgl[k], ws = wk - wg;
-    if (std::is_same<T, float>::value && !G.dbg_fstar) {
-      // FP32 storage: the wall distribution and the ghost value of the step
-      // in FP32 (the wall density above stays FP64; a launch that reports
-      // f*_w for the wall quantities takes the FP64 branch below, so that
-      // the normal mass flux of f*_w vanishes to FP64 rounding)
-      const float wkf = (float)wk, wgf = (float)wg, wsf = wkf - wgf, rw = (float)G.rwD[k];
-      const float arw = (float)(alpha * rho_w), oma = (float)(1.0 - alpha), cgc = (float)c_gc, Gwf = (float)Gw;
-#pragma unroll
-      for (int m = 0; m < NC; ++m) {
-        const size_t o = ((size_t)l * G.nvp + k) * NC + m;
-        const float gw = (m == 0) ? Gwf : (float)(0.5 * G.Tw) * Gwf;
-        const float fr = arw * gw + oma * (float)fsv[m];
-        const float fiv = (float)G.fi[o];
-        const float fstar = (wkf > 0.f) ? (wgf * fiv + wsf * fr) * rw : fiv;
-        const float spv = (float)G.fsp[o];
-        float gv = spv + cgc * (fstar - spv);
-        if (G.ghost_nonneg && gv < 0.f) gv = 0.f;
-        G.lval[o] = (T)gv;
       }
-      continue;
-    }
-#pragma unroll
-    for (int m = 0; m < NC; ++m) {
-      const size_t o = ((size_t)l * G.nvp + k) * NC + m;
-      const double gw = (m == 0) ? Gw : 0.5 * G.Tw * Gw; // B_w = T_w / 2 H_w
-      const double fr = alpha * rho_w * gw + (1.0 - alpha) * fsv[m];
-      const double fiv = (double)G.fi[o];
-      const double fstar = (wk > 0.0) ? (wg * fiv + ws * fr) * G.rwD[k] : fiv;
-      const double spv = (double)G.fsp[o];
-      double gv = spv + c_gc * (fstar - spv);
-      if (G.ghost_nonneg && gv < 0.0) gv = 0.0; // optional nonnegative ghost values
-      G.lval[o] = (T)gv;
-      if (G.dbg_fstar) G.dbg_fstar[o] = fstar;
-    }
+    cluster_sums<NQ>(S, nq, sh, s_sum[1]);
   }
+#pragma unroll
+  for (int q = 0; q < NQ; ++q)
+    if (q < nq) {
+      const int l = l0 + q;
+      const double *ld = G.l_dbl + 8 * l;
+      const double c_gc = ld[2], nw[3] = {ld[3], ld[4], ld[5]};
+      // ld[7]: the reflected mass flux per unit wall density (geometry and wall only)
+      const double rho_w = (alpha > 0.0) ? -(N[q] + (1.0 - alpha) * S[q]) / (alpha * ld[7]) : 0.0;
+      if (rank == 0 && threadIdx.x == 0) G.rhow[l] = rho_w;
+      // wall distribution (Eqs. general bc, Maxwell BC, fwc) and ghost value (Eq. extrapolation 2)
+      const T arw = (T)(alpha * rho_w), oma = (T)(1.0 - alpha), cgc = (T)c_gc, halfT = (T)(0.5 * G.Tw);
+#pragma unroll 2
+      for (int k = k0 + threadIdx.x; k < k1; k += kGhostThreads) {
+        double fsv[NC], xn;
+#pragma unroll
+        for (int m = 0; m < NC; ++m) fsv[m] = 0.0;
+        if (alpha < 1.0) mirrored<T, D>(G, l, k, nw, xn, fsv);
+        const size_t o = ((size_t)l * G.nvp + k) * NC;
+        T fi[NC], sp[NC], gv[NC];
+        load_nc<T, NC>(G.fi + o, fi);
+        load_nc<T, NC>(G.fsp + o, sp);
+        if (!G.dbg_fstar) {
+          // the wall distribution and the ghost value of the step in the storage
+          // type (the wall density above stays FP64; a launch that reports f*_w for
+          // the wall quantities takes the FP64 branch below, so that the normal
+          // mass flux of f*_w vanishes to FP64 rounding)
+          const T al = G.l_al[(size_t)l * G.nvp + k], Gw = G.gwT[k];
+#pragma unroll
+          for (int m = 0; m < NC; ++m) {
+            const T fr = arw * ((m == 0) ? Gw : halfT * Gw) + oma * (T)fsv[m];
+            const T fstar = al * fi[m] + (T(1) - al) * fr;
+            gv[m] = sp[m] + cgc * (fstar - sp[m]);
+            if (G.ghost_nonneg && gv[m] < T(0)) gv[m] = T(0); // optional nonnegative ghost values
+          }
+        } else {
+          const double wk = G.wD[k], wg = G.l_wg[(size_t)l * G.nvp + k], ws = wk - wg, Gw = G.gwu[k];
+#pragma unroll
+          for (int m = 0; m < NC; ++m) {
+            const double gw = (m == 0) ? Gw : 0.5 * G.Tw * Gw; // B_w = T_w / 2 H_w
+            const double fr = alpha * rho_w * gw + (1.0 - alpha) * fsv[m];
+            const double fiv = (double)fi[m], spv = (double)sp[m];
+            const double fstar = (wk > 0.0) ? (wg * fiv + ws * fr) * G.rwD[k] : fiv;
+            double v = spv + c_gc * (fstar - spv);
+            if (G.ghost_nonneg && v < 0.0) v = 0.0;
+            gv[m] = (T)v;
+            G.dbg_fstar[o + m] = fstar;
+          }
+        }
+        store_nc<T, NC>(G.lval + o, gv);
+      }
+    }
+  cl.sync(); // no block leaves while another may read its sums
+}
+
+// The link tables that depend on the geometry and the wall only: per link and
+// velocity the incident mass flux per unit f and the incident share of the
+// velocity's box, per link the reflected mass flux per unit wall density
+// (FP64; one block per link, when a body is set).
+template <typename T, int D>
+__global__ void __launch_bounds__(256) ghost_tables_kernel(GhostArgs<T> G, double *l_dbl, double *l_cn, T *l_al) {
+  __shared__ double sh[256 / 32 + 1];
+  const int l = blockIdx.x;
+  double *ld = l_dbl + 8 * l;
+  double Dsum = 0.0;
+  for (int k = threadIdx.x; k < G.nvp; k += blockDim.x) {
+    const size_t o = (size_t)l * G.nvp + k;
+    double xn = 0.0;
+    for (int a = 0; a < D; ++a) xn += G.xiD[a * G.nvp + k] * ld[3 + a];
+    const double w = G.wD[k], wg = G.l_wg[o];
+    l_cn[o] = wg * xn;
+    l_al[o] = (w > 0.0) ? (T)(wg * G.rwD[k]) : T(1);
+    Dsum += (w - wg) * xn * G.gwu[k];
+  }
+  Dsum = block_sum<256>(Dsum, sh);
+  if (threadIdx.x == 0) ld[7] = Dsum;
 }
 
 template <typename T, int D>
-__global__ void __launch_bounds__(kGhostThreads, (GhostTiling<T, false>::blocks)) ghost_band_kernel(GhostArgs<T> G) {
-  ghost_band_body<T, D, GhostTiling<T, false>::U>(G, blockIdx.x);
+__global__ void __launch_bounds__(kGhostThreads) ghost_band_kernel(const __grid_constant__ GhostArgs<T> G) {
+  ghost_band_body<T, D>(G, blockIdx.x / cooperative_groups::this_cluster().num_blocks());
+}
+
+// a launch of the ghost band's kernels: clusters of `split` blocks
+template <typename... A, typename... B>
+cudaError_t launch_clusters(void (*fn)(A...), int clusters, int split, cudaStream_t s, B... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)clusters * split);
+  cfg.blockDim = dim3(kGhostThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = split;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
 // ---------------------------------------------------------------------------
@@ -1801,19 +1927,23 @@ template <typename T> struct ForceArgs {
   const int *__restrict__ l_int;
   const double *__restrict__ l_dbl;
   const double *__restrict__ xiD;
-  const double *__restrict__ wD;
-  double *__restrict__ fpart; // [nlink][4]
+  const double *__restrict__ wxi; // [4][nvp]: w xi_x, w xi_y, w xi_z, |xi|^2 / 2
+  double *__restrict__ fpart; // [nlink][kForceSplit][4]
   int nlink;
   double *__restrict__ dst;   // [4]: F_x, F_y, F_z, Q
+  int *__restrict__ count;    // blocks of the launch done (zero between launches)
   // a tree (C29): per link the row beyond the donor along the link axis (a
   // leaf, -2 the halo, -3 - l the ghost value of link l); null on uniform grids
   const int *__restrict__ tree_far;
 };
 
+// One of kForceSplit blocks of link l: its share of the velocities.  The last
+// block of the member (of nlink kForceSplit) adds all shares in a fixed order.
 template <typename T, int D>
-__device__ __forceinline__ void forces_body(const ForceArgs<T> &A, const int l) {
+__device__ __forceinline__ void forces_body(const ForceArgs<T> &A, const int l, const int rank) {
   constexpr int NC = Dims<D>::NC;
-  __shared__ double sh[16];
+  __shared__ double sh[4][kForceThreads / 32];
+  __shared__ bool s_last;
   const int *li = A.l_int + 8 * l;
   const int d = li[1], a = li[3], side = li[4];
   const int sf = -side; // face of the donor toward the ghost
@@ -1823,71 +1953,85 @@ __device__ __forceinline__ void forces_body(const ForceArgs<T> &A, const int l) 
   ijk[0] = d % S.n[0];
   ijk[1] = (d / S.n[0]) % S.n[1];
   ijk[2] = d / (S.n[0] * S.n[1]);
+  // the rows of the donor, the link's ghost value, and the value beyond the donor
+  const T *fdr = S.f + (size_t)d * S.nvp * NC, *fgr = S.lval + (size_t)l * S.nvp * NC, *fbr;
+  if (A.tree_far) {
+    const int r = A.tree_far[l];
+    fbr = (r >= 0) ? S.f + (size_t)r * S.nvp * NC : (r == -2) ? S.finf : S.lval + (size_t)(-3 - r) * S.nvp * NC;
+  } else {
+    fbr = seen_row<T, NC>(S, d, ijk, a, -sf);
+  }
   double acc[4] = {0, 0, 0, 0};
-  for (int iv = threadIdx.x; iv < S.nv; iv += blockDim.x) {
-    const int k = S.kst[iv];
-    const double xin = A.xiD[a * S.nvp + k] * sf; // velocity into the solid
-    if (xin == 0.0) continue;
-    T fd[NC], fg[NC], face[NC];
-    load_nc<T, NC>(S.f + ((size_t)d * S.nvp + k) * NC, fd);
-    if (A.tree_far) load_nc<T, NC>(S.lval + ((size_t)l * S.nvp + k) * NC, fg);
-    else seen<T, NC>(S, d, ijk, a, sf, k, fg); // the link's ghost value
-    if (xin > 0.0) {
-      T fb[NC];
-      if (A.tree_far) {
-        const int r = A.tree_far[l];
-        load_nc<T, NC>((r >= 0) ? S.f + ((size_t)r * S.nvp + k) * NC
-                       : (r == -2) ? S.finf + (size_t)k * NC : S.lval + ((size_t)(-3 - r) * S.nvp + k) * NC, fb);
-      } else {
-        seen<T, NC>(S, d, ijk, a, -sf, k, fb);
-      }
+  const double *wxa = A.wxi + (size_t)a * S.nvp, *x2 = A.wxi + 3 * (size_t)S.nvp;
+  constexpr int U = 4; // velocities of a thread at a time: their loads are in flight together
+  for (int kb = rank * kForceThreads + threadIdx.x; kb < S.nvp; kb += U * kForceSplit * kForceThreads) {
+    T fd[U][NC], fg[U][NC], fb[U][NC], xin[U];
+    double wa[U], xb[U][D], xx[U];
 #pragma unroll
-      for (int m = 0; m < NC; ++m) face[m] = fd[m] + T(0.5) * vanleer(fd[m] - fb[m], fg[m] - fd[m]);
-    } else {
+    for (int u = 0; u < U; ++u) {
+      const int kq = kb + u * kForceSplit * kForceThreads;
+      const bool ok = kq < S.nvp;
+      const int k = ok ? kq : kb;
+      xin[u] = ok ? S.xi[a * S.nvp + k] * T(sf) : T(0); // velocity into the solid (zero at padding positions)
+      load_nc<T, NC>(fdr + (size_t)k * NC, fd[u]);
+      load_nc<T, NC>(fgr + (size_t)k * NC, fg[u]);
+      load_nc<T, NC>(fbr + (size_t)k * NC, fb[u]);
+      wa[u] = wxa[k];
+      xx[u] = x2[k];
 #pragma unroll
-      for (int m = 0; m < NC; ++m) face[m] = T(0.5) * (fg[m] + fd[m]);
+      for (int b = 0; b < D; ++b) xb[u][b] = A.xiD[b * S.nvp + k];
     }
-    const double wk = A.wD[k];
-    double x2 = 0.0;
-    for (int b = 0; b < D; ++b) {
-      const double x = A.xiD[b * S.nvp + k];
-      x2 += x * x;
-      acc[b] += Sface * wk * x * xin * (double)face[0];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (xin[u] == T(0)) continue;
+      T face[NC];
+#pragma unroll
+      for (int m = 0; m < NC; ++m)
+        face[m] = (xin[u] > T(0)) ? fd[u][m] + T(0.5) * vanleer(fd[u][m] - fb[u][m], fg[u][m] - fd[u][m])
+                                  : T(0.5) * (fg[u][m] + fd[u][m]);
+      // FP64 sums; the face's area and side enter at the end
+      const double t = wa[u] * (double)face[0];
+#pragma unroll
+      for (int b = 0; b < D; ++b) acc[b] += xb[u][b] * t;
+      acc[3] += xx[u] * t;
+      if (D == 2) acc[3] += (0.5 * wa[u]) * (double)face[NC - 1];
     }
-    double e = 0.5 * x2 * (double)face[0];
-    if (D == 2) e += 0.5 * (double)face[NC - 1];
-    acc[3] += Sface * wk * e * xin;
   }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
   for (int i = 0; i < 4; ++i) {
-    double s = block_sum<256>(acc[i], sh);
-    if (threadIdx.x == 0) A.fpart[4 * l + i] = s;
+    double v = acc[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) sh[i][wid] = v;
   }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    double v = 0.0;
+    for (int w = 0; w < kForceThreads / 32; ++w) v += sh[threadIdx.x][w];
+    A.fpart[4 * ((size_t)l * kForceSplit + rank) + threadIdx.x] = v * (Sface * sf);
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(A.count, 1) == A.nlink * kForceSplit - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // thread t adds every 32nd share of component t / 32, then the warp its lanes
+  const int n = A.nlink * kForceSplit;
+  double v = 0.0;
+  for (int q = lane; q < n; q += 32) v += __ldcg(A.fpart + 4 * (size_t)q + wid);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if (lane == 0) A.dst[wid] = v;
+  if (threadIdx.x == 0) *A.count = 0;
 }
+static_assert(kForceThreads == 128, "one warp per force component in the last block");
+static_assert(4 * kForceSplit == kForceParts, "partial sums of a link");
 
 template <typename T, int D>
-__global__ void __launch_bounds__(256) forces_kernel(ForceArgs<T> A) {
-  forces_body<T, D>(A, blockIdx.x);
-}
-
-__device__ __forceinline__ void forces_total_body(const double *__restrict__ fpart, int nlink,
-                                                  double *__restrict__ out) {
-  __shared__ double sh[256];
-  for (int i = 0; i < 4; ++i) {
-    double s = 0.0;
-    for (int l = threadIdx.x; l < nlink; l += blockDim.x) s += fpart[4 * l + i];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[i] = sh[0];
-    __syncthreads();
-  }
-}
-
-__global__ void forces_total_kernel(const double *__restrict__ fpart, int nlink, double *__restrict__ out) {
-  forces_total_body(fpart, nlink, out);
+__global__ void __launch_bounds__(kForceThreads) forces_kernel(const __grid_constant__ ForceArgs<T> A) {
+  forces_body<T, D>(A, blockIdx.x / kForceSplit, blockIdx.x % kForceSplit);
 }
 
 // ---------------------------------------------------------------------------
@@ -1908,29 +2052,35 @@ __device__ __forceinline__ int group_case(const int *__restrict__ start, int nca
 }
 
 template <typename T, int D>
-__global__ void __launch_bounds__(kGhostThreads, (GhostTiling<T, true>::blocks)) ghost_band_grouped(const GhostArgs<T> *__restrict__ tab,
-                                                          const int *__restrict__ start, int ncase, int par) {
+__global__ void __launch_bounds__(kGhostThreads)
+    surface_slopes_grouped(const GhostArgs<T> *__restrict__ tab, const int *__restrict__ start, int ncase, int par) {
   __shared__ GhostArgs<T> sG;
   const int c = group_case(start, ncase, blockIdx.x);
   if (threadIdx.x == 0) sG = tab[2 * c + par];
   __syncthreads();
-  ghost_band_body<T, D, GhostTiling<T, true>::U>(sG, blockIdx.x - __ldg(start + c));
+  surface_slopes_body<T, D>(sG, blockIdx.x - __ldg(start + c));
 }
 
 template <typename T, int D>
-__global__ void __launch_bounds__(256) forces_grouped(const ForceArgs<T> *__restrict__ tab,
-                                                      const int *__restrict__ start, int ncase, int par) {
-  __shared__ ForceArgs<T> sA;
-  const int c = group_case(start, ncase, blockIdx.x);
-  if (threadIdx.x == 0) sA = tab[2 * c + par];
+__global__ void __launch_bounds__(kGhostThreads)
+    ghost_band_grouped(const GhostArgs<T> *__restrict__ tab, const int *__restrict__ start, int ncase, int par) {
+  __shared__ GhostArgs<T> sG;
+  const int vg = blockIdx.x / cooperative_groups::this_cluster().num_blocks();
+  const int c = group_case(start, ncase, vg);
+  if (threadIdx.x == 0) sG = tab[2 * c + par];
   __syncthreads();
-  forces_body<T, D>(sA, blockIdx.x - __ldg(start + c));
+  ghost_band_body<T, D>(sG, vg - __ldg(start + c));
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) forces_total_grouped(const ForceArgs<T> *__restrict__ tab, int par) {
-  const ForceArgs<T> &A = tab[2 * blockIdx.x + par];
-  forces_total_body(A.fpart, A.nlink, A.dst);
+template <typename T, int D>
+__global__ void __launch_bounds__(kForceThreads) forces_grouped(const ForceArgs<T> *__restrict__ tab,
+                                                                const int *__restrict__ start, int ncase, int par) {
+  __shared__ ForceArgs<T> sA;
+  const int vl = blockIdx.x / kForceSplit;
+  const int c = group_case(start, ncase, vl);
+  if (threadIdx.x == 0) sA = tab[2 * c + par];
+  __syncthreads();
+  forces_body<T, D>(sA, vl - __ldg(start + c), blockIdx.x % kForceSplit);
 }
 
 template <typename T, int D, typename P>
@@ -2108,9 +2258,16 @@ template <typename T> GhostArgs<T> ghost_args(const ibdvm_ctx *ctx, int cur, dou
   G.l_int = ctx->l_int;
   G.l_dbl = ctx->l_dbl;
   G.l_wg = ctx->l_wg;
-  G.s_int = ctx->s_int;
-  G.s_dbl = ctx->s_dbl;
+  G.l_cn = ctx->l_cn;
+  G.l_al = static_cast<const T *>(ctx->l_al);
+  G.g_int = ctx->g_int;
+  G.e_int = ctx->e_int;
+  G.c_int = ctx->c_int;
+  G.s_T = static_cast<const T *>(ctx->s_T);
+  G.sig = static_cast<T *>(ctx->sig);
+  G.split = ghost_split(ctx->nvp);
   G.gwu = ctx->gw_unit;
+  G.gwT = static_cast<const T *>(ctx->gw_T);
   G.kst = ctx->kst;
   G.lval = static_cast<T *>(ctx->lval);
   G.fi = static_cast<T *>(ctx->fi_scr);
@@ -2167,10 +2324,18 @@ template <typename T, int D> cudaError_t domain_t(ibdvm_ctx *ctx) {
   return cudaGetLastError();
 }
 
+// blocks of the slope kernel
+inline int slope_blocks(const ibdvm_ctx *ctx) { return ctx->nsc * ((ctx->nvp + kSlopeVel - 1) / kSlopeVel); }
+
 template <typename T, int D> cudaError_t ghost_t(ibdvm_ctx *ctx, double *dbg) {
   if (ctx->nlink == 0) return cudaSuccess;
-  ghost_band_kernel<T, D><<<ctx->nlink, kGhostThreads, 0, ctx->stream>>>(ghost_args<T>(ctx, ctx->cur, dbg));
-  return cudaGetLastError();
+  const GhostArgs<T> G = ghost_args<T>(ctx, ctx->cur, dbg);
+  if (!G.naive && ctx->nsc > 0) {
+    surface_slopes_kernel<T, D><<<slope_blocks(ctx), kGhostThreads, 0, ctx->stream>>>(G);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return launch_clusters(ghost_band_kernel<T, D>, ctx->nghost, ghost_split(ctx->nvp), ctx->stream, G);
 }
 
 // arguments of the force kernels for state buffer parity cur
@@ -2180,20 +2345,18 @@ template <typename T> ForceArgs<T> force_args(const ibdvm_ctx *ctx, int cur, dou
   A.l_int = ctx->l_int;
   A.l_dbl = ctx->l_dbl;
   A.xiD = ctx->xiD;
-  A.wD = ctx->wD;
+  A.wxi = ctx->wD + 2 * (size_t)ctx->nvp;
   A.fpart = ctx->fpart;
   A.nlink = ctx->nlink;
   A.dst = dst;
+  A.count = ctx->fcount;
   A.tree_far = ctx->tree ? ctx->tree_far : nullptr;
   return A;
 }
 
 template <typename T, int D> cudaError_t forces_t(ibdvm_ctx *ctx, double *dst) {
   if (ctx->nlink == 0) return cudaMemsetAsync(dst, 0, 4 * sizeof(double), ctx->stream);
-  forces_kernel<T, D><<<ctx->nlink, 256, 0, ctx->stream>>>(force_args<T>(ctx, ctx->cur, dst));
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  forces_total_kernel<<<1, 256, 0, ctx->stream>>>(ctx->fpart, ctx->nlink, dst);
+  forces_kernel<T, D><<<ctx->nlink * kForceSplit, kForceThreads, 0, ctx->stream>>>(force_args<T>(ctx, ctx->cur, dst));
   return cudaGetLastError();
 }
 
@@ -2316,7 +2479,7 @@ cudaError_t launch_ghost_band(ibdvm_ctx *ctx, double *dbg) {
   Timed t(ctx, kKGhost);
   // the halo values of diffuse domain walls first: the pre-ghost slopes and
   // the sweep read them
-  ctx->kernel_launches[kKGhost] += (ctx->wall_mask ? 1 : 0) + (ctx->nlink ? 1 : 0);
+  ctx->kernel_launches[kKGhost] += (ctx->wall_mask ? 1 : 0) + (ctx->nlink ? 2 : 0);
   return dispatch(ctx, [&](auto t, auto d) -> cudaError_t {
     using T = decltype(t);
     constexpr int D = decltype(d)::value;
@@ -2325,6 +2488,17 @@ cudaError_t launch_ghost_band(ibdvm_ctx *ctx, double *dbg) {
       if (e != cudaSuccess) return e;
     }
     return ghost_t<T, D>(ctx, dbg);
+  });
+}
+
+cudaError_t launch_ghost_tables(ibdvm_ctx *ctx) {
+  if (ctx->nlink == 0) return cudaSuccess;
+  return dispatch(ctx, [&](auto t, auto d) -> cudaError_t {
+    using T = decltype(t);
+    constexpr int D = decltype(d)::value;
+    ghost_tables_kernel<T, D><<<ctx->nlink, 256, 0, ctx->stream>>>(ghost_args<T>(ctx, ctx->cur, nullptr), ctx->l_dbl,
+                                                                  ctx->l_cn, static_cast<T *>(ctx->l_al));
+    return cudaGetLastError();
   });
 }
 
@@ -2381,7 +2555,7 @@ cudaError_t launch_sweep(ibdvm_ctx *ctx) {
 
 cudaError_t launch_forces(ibdvm_ctx *ctx, double *dst) {
   Timed t(ctx, kKForces);
-  ctx->kernel_launches[kKForces] += ctx->nlink ? 2 : 0;
+  ctx->kernel_launches[kKForces] += ctx->nlink ? 1 : 0;
   return dispatch(ctx, [&](auto t, auto d) -> cudaError_t {
     using T = decltype(t);
     constexpr int D = decltype(d)::value;
@@ -2420,7 +2594,7 @@ template <typename T> cudaError_t upload_table(const std::vector<T> &h, void *&d
 } // namespace
 
 void group_free(GroupTables &t) {
-  void *ps[] = {t.ghost, t.force, t.fin, t.link_start, t.fin_start};
+  void *ps[] = {t.ghost, t.force, t.fin, t.link_start, t.ghost_start, t.slope_start, t.fin_start};
   for (void *p : ps)
     if (p) cudaFree(p);
   t = GroupTables{};
@@ -2432,13 +2606,17 @@ cudaError_t group_build(const std::vector<ibdvm_ctx *> &cases, const std::vector
   const int n = static_cast<int>(cases.size());
   t.ncase = n;
   t.dim = n ? cases[0]->dim : 2;
-  std::vector<int> ls(n + 1, 0), fs(n + 1, 0);
+  std::vector<int> ls(n + 1, 0), gs(n + 1, 0), ss(n + 1, 0), fs(n + 1, 0);
+  t.split = 1;
   std::vector<GhostArgs<float>> g(2 * n);
   std::vector<ForceArgs<float>> fa(2 * n);
   std::vector<FinalArgs<float, float>> fi(2 * n);
   for (int i = 0; i < n; ++i) {
     const ibdvm_ctx *ctx = cases[i];
     ls[i + 1] = ls[i] + ctx->nlink;
+    gs[i + 1] = gs[i] + (ctx->nlink ? ctx->nghost : 0);
+    ss[i + 1] = ss[i] + (ctx->nlink ? slope_blocks(ctx) : 0);
+    t.split = std::max(t.split, ghost_split(ctx->nvp));
     fs[i + 1] = fs[i] + static_cast<int>((ctx->ncell + 255) / 256);
     for (int p = 0; p < 2; ++p) {
       g[2 * i + p] = ghost_args<float>(ctx, ctx->cur ^ p, nullptr);
@@ -2450,6 +2628,8 @@ cudaError_t group_build(const std::vector<ibdvm_ctx *> &cases, const std::vector
     }
   }
   t.link_blocks = ls[n];
+  t.ghost_blocks = gs[n];
+  t.slope_blocks = ss[n];
   t.fin_blocks = fs[n];
   cudaError_t e;
   if ((e = upload_table(g, t.ghost, s)) != cudaSuccess) return e;
@@ -2458,33 +2638,38 @@ cudaError_t group_build(const std::vector<ibdvm_ctx *> &cases, const std::vector
   void *p0 = nullptr, *p1 = nullptr;
   if ((e = upload_table(ls, p0, s)) != cudaSuccess) return e;
   t.link_start = static_cast<int *>(p0);
+  if ((e = upload_table(gs, p0, s)) != cudaSuccess) return e;
+  t.ghost_start = static_cast<int *>(p0);
+  if ((e = upload_table(ss, p0, s)) != cudaSuccess) return e;
+  t.slope_start = static_cast<int *>(p0);
   if ((e = upload_table(fs, p1, s)) != cudaSuccess) return e;
   t.fin_start = static_cast<int *>(p1);
   return cudaStreamSynchronize(s); // the host tables go out of scope
 }
 
 cudaError_t group_ghost(const GroupTables &t, int par, cudaStream_t s) {
-  if (t.link_blocks == 0) return cudaSuccess;
+  if (t.ghost_blocks == 0) return cudaSuccess;
   const auto *tab = static_cast<const GhostArgs<float> *>(t.ghost);
-  if (t.dim == 2)
-    ghost_band_grouped<float, 2><<<t.link_blocks, kGhostThreads, 0, s>>>(tab, t.link_start, t.ncase, par);
-  else
-    ghost_band_grouped<float, 3><<<t.link_blocks, kGhostThreads, 0, s>>>(tab, t.link_start, t.ncase, par);
-  return cudaGetLastError();
+  if (t.slope_blocks > 0) {
+    if (t.dim == 2)
+      surface_slopes_grouped<float, 2><<<t.slope_blocks, kGhostThreads, 0, s>>>(tab, t.slope_start, t.ncase, par);
+    else
+      surface_slopes_grouped<float, 3><<<t.slope_blocks, kGhostThreads, 0, s>>>(tab, t.slope_start, t.ncase, par);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  const int *start = t.ghost_start;
+  return (t.dim == 2) ? launch_clusters(ghost_band_grouped<float, 2>, t.ghost_blocks, t.split, s, tab, start, t.ncase, par)
+                      : launch_clusters(ghost_band_grouped<float, 3>, t.ghost_blocks, t.split, s, tab, start, t.ncase, par);
 }
 
 cudaError_t group_forces(const GroupTables &t, int par, cudaStream_t s) {
-  if (t.ncase == 0) return cudaSuccess;
+  if (t.link_blocks == 0) return cudaSuccess; // a member without links keeps its zeros
   const auto *tab = static_cast<const ForceArgs<float> *>(t.force);
-  if (t.link_blocks > 0) {
-    if (t.dim == 2)
-      forces_grouped<float, 2><<<t.link_blocks, 256, 0, s>>>(tab, t.link_start, t.ncase, par);
-    else
-      forces_grouped<float, 3><<<t.link_blocks, 256, 0, s>>>(tab, t.link_start, t.ncase, par);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  forces_total_grouped<float><<<t.ncase, 256, 0, s>>>(tab, par);
+  if (t.dim == 2)
+    forces_grouped<float, 2><<<t.link_blocks * kForceSplit, kForceThreads, 0, s>>>(tab, t.link_start, t.ncase, par);
+  else
+    forces_grouped<float, 3><<<t.link_blocks * kForceSplit, kForceThreads, 0, s>>>(tab, t.link_start, t.ncase, par);
   return cudaGetLastError();
 }
 
