@@ -717,7 +717,7 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
       // the threads of a warp of the tree sweep share upwind sides
       int pos = 0;
       for (int o = 0; o < (1 << G.dim); ++o) {
-        if (o > 0 && o < 4) ctx->tree_qb[o - 1] = pos;
+        if (o > 0) ctx->tree_qb[o - 1] = pos;
         for (int i = 0; i < G.nv; ++i) {
           int oi = 0;
           for (int a = 0; a < G.dim; ++a) oi |= (G.xi[3 * i + a] < 0.0) ? (1 << a) : 0;

@@ -170,7 +170,7 @@ struct ibdvm_ctx {
   std::vector<int> tree_lev_h, tree_own; // leaf levels; the leaf of every finest-grid cell
   ibdvm::Geom tree_vgeom;                // the finest grid (a body is placed there)
   int *tree_far = nullptr;               // [link] row beyond the donor (map_tree_body)
-  int tree_qb[3] = {0, 0, 0}; // first stored velocity of the quadrants 1, 2, 3 (bit 0: x < 0, bit 1: y < 0)
+  int tree_qb[7] = {}; // first stored velocity of the orthants 1 .. 2^dim - 1 (bit a: component a < 0)
   std::vector<int> tree_nb_h;
   // host uploads of the state in cell ranges (a copy stream, one event per range)
   cudaStream_t copy_stream = nullptr;
@@ -197,6 +197,8 @@ cudaError_t launch_wall(ibdvm_ctx *ctx, const double *fstar, double *out);
 cudaError_t launch_ghost_band(ibdvm_ctx *ctx, double *dbg_fstarw);
 cudaError_t launch_sweep(ibdvm_ctx *ctx);
 cudaError_t launch_forces(ibdvm_ctx *ctx, double *dst);
+// the sweep of a tree in FP32 storage (tree_sweep.cu)
+cudaError_t tree_sweep32_launch(ibdvm_ctx *ctx);
 // the ghost band's tables of the geometry and the wall (after a body is uploaded)
 cudaError_t launch_ghost_tables(ibdvm_ctx *ctx);
 // TMA sweep (sweep_tma.cu)

@@ -431,7 +431,6 @@ template <typename T> struct TreeArgs {
   const double2 *__restrict__ stg;  // [leaf][entries][2]: 1/d-, 1/d+, h, 1/h (own entries)
   const int4 *__restrict__ lrec;    // [leaf][2]: leaves on the sides, regular flag, fluid flag
   const int *__restrict__ sched;    // [leaf]: the leaf of each block slot (regular, other fluid, solid)
-  int qb[3];                        // 2D: first stored position of the quadrants 1, 2, 3 (bit 0: x < 0, bit 1: y < 0)
 };
 
 // the stencil of one cell along one axis: the rows [nvp][NC] of the cell and
@@ -470,14 +469,6 @@ __device__ __forceinline__ void tree_side_value(const T *const *r, int k, T *v) 
   }
 }
 
-// the van Leer limiter of the tree sweep: FP64 divides; FP32 takes the
-// hardware reciprocal (as the packed quadtree path does)
-__device__ __forceinline__ double tree_vanleer(double a, double b) { return vanleer(a, b); }
-__device__ __forceinline__ float tree_vanleer(float a, float b) {
-  const float p = a * b;
-  return (p > 0.f) ? 2.f * p * dev::rcp_approx(a + b) : 0.f;
-}
-
 // the face value on side s of a cell of value fc with side values fm, fp:
 // the limited slope over the centre distances times s h / 2
 template <typename T, int NC, int NF>
@@ -485,7 +476,7 @@ __device__ __forceinline__ void tree_face_value(const TreeStencil<T, NF> &S, con
                                                 T *out) {
   const T sh = s * (T(0.5) * S.h);
 #pragma unroll
-  for (int m = 0; m < NC; ++m) out[m] = fc[m] + tree_vanleer((fc[m] - fm[m]) * S.rdm, (fp[m] - fc[m]) * S.rdp) * sh;
+  for (int m = 0; m < NC; ++m) out[m] = fc[m] + vanleer((fc[m] - fm[m]) * S.rdm, (fp[m] - fc[m]) * S.rdp) * sh;
 }
 
 // the face value of the upwind stencil S on side s (its own value and sides loaded)
@@ -498,38 +489,13 @@ __device__ __forceinline__ void tree_upwind_face(const TreeStencil<T, NF> &S, T 
   tree_face_value<T, NC, NF>(S, fu, um, up, s, out);
 }
 
-// FP32 (h, b) pairs of quadtrees: packed arithmetic, the limiter through the
-// hardware reciprocal (half the van Leer slope times the edge: h ab / (a + b))
-__device__ __forceinline__ float2 tree_side2(const float *r0, const float *r1, int k) {
-  const float2 v = reinterpret_cast<const float2 *>(r0)[k];
-  if (!r1) return v;
-  const float2 w = reinterpret_cast<const float2 *>(r1)[k];
-  return __fmul2_rn(__fadd2_rn(v, w), dev::dup(0.5f));
-}
-__device__ __forceinline__ float2 tree_face2(const TreeStencil<float, 2> &S, float2 fc, float2 fm, float2 fp, float s) {
-  const float2 a = __fmul2_rn(dev::sub2(fc, fm), dev::dup(S.rdm));
-  const float2 b = __fmul2_rn(dev::sub2(fp, fc), dev::dup(S.rdp));
-  return __ffma2_rn(dev::dup(s * S.h), dev::vl_half2(a, b), fc);
-}
-// 2^x (the hardware base-2 exponential)
-__device__ __forceinline__ float tree_ex2(float x) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-constexpr float kTreeLog2e = 1.442695040888963407f;
-
-// FP32: four blocks of 256 threads per SM (the loop waits on gathers from L2
-// and HBM: resident warps hide it, a few spilled registers cost less); FP64,
-// bound by its arithmetic: two
-template <typename T, int D>
-__global__ void __launch_bounds__(kBlock, (sizeof(T) == 4) ? 4 : 2) tree_sweep_kernel(TreeArgs<T> TA) {
+// FP64 storage, bound by its arithmetic (FP32 storage: tree_sweep.cu)
+template <typename T, int D> __global__ void __launch_bounds__(kBlock, 2) tree_sweep_kernel(TreeArgs<T> TA) {
   constexpr int NC = Dims<D>::NC;
   constexpr int NM = Dims<D>::NM;
   constexpr int NF = 1 << (D - 1); // leaves at most beyond a face
   constexpr int NS = 2 * D;        // sides
   constexpr int E = tree_entries(D), EI = tree_entry_ints(D);
-  constexpr bool kF32 = std::is_same<T, float>::value && D == 2; // the packed quadtree paths
   static_assert(E <= kThreadsPerCell, "one thread per stencil entry");
   const SweepArgs<T> &A = TA.S;
   __shared__ double red[kCellsPerBlock][2][NM];
@@ -538,7 +504,6 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4) ? 4 : 2) tree_sweep_k
   __shared__ TreeStencil<T, NF> st[kCellsPerBlock][E];
   __shared__ int nup[kCellsPerBlock][NS]; // leaves on side 2a + sd: 0 (domain edge), 1, NF, 3 (a ghost)
   __shared__ T rh[kCellsPerBlock][D];     // 1 / h
-  __shared__ int fast[kCellsPerBlock];    // one neighbour of the leaf's own level on every side (2D)
   __shared__ int fluid[kCellsPerBlock];   // the leaf is updated (not a solid leaf of a body, C29)
   const int tx = threadIdx.x, ty = threadIdx.y;
   const long long slot = (long long)blockIdx.x * kCellsPerBlock + ty;
@@ -582,7 +547,6 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4) ? 4 : 2) tree_sweep_k
     const int r[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
 #pragma unroll
     for (int s = 0; s < NS; ++s) nup[ty][s] = r[s];
-    fast[ty] = r[NS];
     fluid[ty] = r[NS + 1];
   }
   __syncthreads();
@@ -722,165 +686,6 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4) ? 4 : 2) tree_sweep_k
           c2 += cv[a] * cv[a];
         }
         moments(cv, c2, A.w[k], fc);
-      }
-    } else if constexpr (kF32) {
-      const float nl2 = -invT * kTreeLog2e;
-      const float2 *finf2 = reinterpret_cast<const float2 *>(A.finf);
-      // relaxation, the store of f^{n+1} and the moment sums of one velocity
-      auto finish = [&](int k, float2 f2, float2 dv, const float *cv, float c2, float wk) {
-        // Shakhov equilibrium (Sec. 4 reduced forms)
-        const float cq = fmaf(cv[1], q[1], cv[0] * q[0]);
-        const float e = pre * tree_ex2(c2 * nl2);
-        const float corr = shA * cq;
-        const float tc = 2.f * c2 * invT;
-        const float H = e * fmaf(corr, tc - 4.f, 1.f);
-        const float B = halfT * e * fmaf(corr, tc - 2.f, 1.f);
-        float fo[2];
-        fo[0] = f2.x - A.dt * dv.x + dtau * (H - f2.x);
-        fo[1] = f2.y - A.dt * dv.y + dtau * (B - f2.y);
-        reinterpret_cast<float2 *>(A.fn)[(size_t)c * A.nvp + k] = make_float2(fo[0], fo[1]);
-        // moments about the current bulk velocity: c' = xi - U^n
-        const float wh = wk * fo[0];
-        const float e2 = fmaf(c2, wh, wk * fo[1]);
-        acc[0] += wh;
-        acc[1] = fmaf(cv[0], wh, acc[1]);
-        acc[2] = fmaf(cv[1], wh, acc[2]);
-        acc[3] += e2;
-        acc[4] = fmaf(cv[0] * cv[0], wh, acc[4]);
-        acc[5] = fmaf(cv[0] * cv[1], wh, acc[5]);
-        acc[6] = fmaf(cv[1] * cv[1], wh, acc[6]);
-        acc[7] = fmaf(cv[0], e2, acc[7]);
-        acc[8] = fmaf(cv[1], e2, acc[8]);
-      };
-      if (fast[ty]) {
-        // a leaf with one neighbour of its own level on every side: the
-        // upwind neighbour's value and its side towards the leaf are the
-        // leaf's side value and own value, so one velocity reads the leaf,
-        // its four neighbours and the two far neighbours upwind; every load
-        // is issued before any arithmetic, the upwind sides taken from the
-        // quadrant of the stored position (a zero component moves nothing)
-        const TreeStencil<float, 2> &Sx = st[ty][0], &Sy = st[ty][1];
-        const float2 *xm = reinterpret_cast<const float2 *>(Sx.m[0]), *xp = reinterpret_cast<const float2 *>(Sx.p[0]);
-        const float2 *ym = reinterpret_cast<const float2 *>(Sy.m[0]), *yp = reinterpret_cast<const float2 *>(Sy.p[0]);
-        const float2 *xf0 = reinterpret_cast<const float2 *>(st[ty][2].m[0]);
-        const float2 *xf1 = reinterpret_cast<const float2 *>(st[ty][4].p[0]);
-        const float2 *yf0 = reinterpret_cast<const float2 *>(st[ty][6].m[0]);
-        const float2 *yf1 = reinterpret_cast<const float2 *>(st[ty][8].p[0]);
-        const float2 *own2 = reinterpret_cast<const float2 *>(own);
-        for (int k = kbeg + tx; k < kend; k += kThreadsPerCell) {
-          const int o = (k >= TA.qb[0]) + (k >= TA.qb[1]) + (k >= TA.qb[2]); // bit 0: x < 0, bit 1: y < 0
-          const int bx = o & 1, by = o >> 1;
-          const float2 f2 = own2[k], vxm = xm[k], vxp = xp[k], vym = ym[k], vyp = yp[k];
-          const float2 vxf = (bx ? xf1 : xf0)[k], vyf = (by ? yf1 : yf0)[k];
-          const float xix = A.xi[k], xiy = A.xi[A.nvp + k], wk = A.w[k];
-          const float sx = bx ? -1.f : 1.f, sy = by ? -1.f : 1.f;
-          const float2 foutx = tree_face2(Sx, f2, vxm, vxp, sx);
-          const float2 fouty = tree_face2(Sy, f2, vym, vyp, sy);
-          const float2 finx = tree_face2(st[ty][bx ? 4 : 2], bx ? vxp : vxm, bx ? f2 : vxf, bx ? vxf : f2, sx);
-          const float2 finy = tree_face2(st[ty][by ? 8 : 6], by ? vyp : vym, by ? f2 : vyf, by ? vyf : f2, sy);
-          float2 dv = __fmul2_rn(dev::dup(fabsf(xix) * rh[ty][0]), dev::sub2(foutx, finx));
-          dv = __ffma2_rn(dev::dup(fabsf(xiy) * rh[ty][1]), dev::sub2(fouty, finy), dv);
-          const float cv[2] = {xix - U[0], xiy - U[1]};
-          finish(k, f2, dv, cv, fmaf(cv[1], cv[1], cv[0] * cv[0]), wk);
-        }
-      } else {
-      for (int k = kbeg + tx; k < kend; k += kThreadsPerCell) {
-        const float2 f2 = reinterpret_cast<const float2 *>(own)[k];
-        float2 dv = make_float2(0.f, 0.f);
-        float cv[2], c2 = 0.f;
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-          const float xa = A.xi[a * A.nvp + k];
-          cv[a] = xa - U[a];
-          c2 = fmaf(cv[a], cv[a], c2);
-          if (xa == 0.f) continue;
-          const float s = (xa > 0.f) ? 1.f : -1.f; // the downwind side
-          const int sd = (xa > 0.f) ? 0 : 1;       // the upwind side
-          const TreeStencil<float, 2> &So = st[ty][a];
-          const float2 fm = tree_side2(So.m[0], So.m[1], k), fp = tree_side2(So.p[0], So.p[1], k);
-          const float2 fout = tree_face2(So, f2, fm, fp, s);
-          const int n = nup[ty][2 * a + sd];
-          float2 fin;
-          if (n == 0) {
-            fin = finf2[k]; // the halo: its value, zero slope
-          } else if (n == 3) {
-            // a ghost upwind (C29): its link value with the one-sided slope
-            const float2 g = reinterpret_cast<const float2 *>(st[ty][2 + 4 * a + 2 * sd].c)[k];
-            fin = __fmul2_rn(__fadd2_rn(g, f2), dev::dup(0.5f));
-          } else {
-            const TreeStencil<float, 2> &S0 = st[ty][2 + 4 * a + 2 * sd];
-            if (S0.mut) {
-              const float2 fu = sd ? fp : fm;
-              const float2 far = sd ? tree_side2(S0.p[0], S0.p[1], k) : tree_side2(S0.m[0], S0.m[1], k);
-              fin = tree_face2(S0, fu, sd ? f2 : far, sd ? far : f2, s);
-            } else {
-              fin = tree_face2(S0, reinterpret_cast<const float2 *>(S0.c)[k], tree_side2(S0.m[0], S0.m[1], k),
-                               tree_side2(S0.p[0], S0.p[1], k), s);
-              if (n == 2) {
-                const TreeStencil<float, 2> &S1 = st[ty][3 + 4 * a + 2 * sd];
-                const float2 g1 = tree_face2(S1, reinterpret_cast<const float2 *>(S1.c)[k],
-                                             tree_side2(S1.m[0], S1.m[1], k), tree_side2(S1.p[0], S1.p[1], k), s);
-                fin = __fmul2_rn(__fadd2_rn(fin, g1), dev::dup(0.5f));
-              }
-            }
-          }
-          dv = __ffma2_rn(dev::dup(fabsf(xa) * rh[ty][a]), dev::sub2(fout, fin), dv);
-        }
-        finish(k, f2, dv, cv, c2, A.w[k]);
-      }
-      }
-    } else if constexpr (D == 3 && std::is_same<T, float>::value) {
-      if (fast[ty]) {
-        // an octree leaf with one fluid neighbour of its own level on every
-        // side: one velocity reads the leaf, its six neighbours and the three
-        // far neighbours upwind (the mutual shortcut), every load before any
-        // arithmetic
-        const T *nm[3], *np[3], *fm0[3], *fp1[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          nm[a] = st[ty][a].m[0];
-          np[a] = st[ty][a].p[0];
-          fm0[a] = st[ty][D + (2 * a) * NF].m[0];     // beyond the - neighbour
-          fp1[a] = st[ty][D + (2 * a + 1) * NF].p[0]; // beyond the + neighbour
-        }
-        for (int k = kbeg + tx; k < kend; k += kThreadsPerCell) {
-          T xa[3], vm[3], vp[3], vf[3];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) xa[a] = A.xi[a * A.nvp + k];
-          const T fc = own[k];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            vm[a] = nm[a][k];
-            vp[a] = np[a][k];
-            vf[a] = (xa[a] > T(0)) ? fm0[a][k] : fp1[a][k];
-          }
-          T cv[3], c2 = T(0), div = T(0);
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            cv[a] = xa[a] - U[a];
-            c2 += cv[a] * cv[a];
-            const bool pos = xa[a] > T(0);
-            const T s = pos ? T(1) : T(-1);
-            const TreeStencil<T, NF> &So = st[ty][a];
-            const TreeStencil<T, NF> &Su = st[ty][D + (2 * a + (pos ? 0 : 1)) * NF];
-            const T fout = fc + tree_vanleer((fc - vm[a]) * So.rdm, (vp[a] - fc) * So.rdp) * (s * (T(0.5) * So.h));
-            const T fu = pos ? vm[a] : vp[a];
-            const T um = pos ? vf[a] : fc, up = pos ? fc : vf[a];
-            const T fin = fu + tree_vanleer((fu - um) * Su.rdm, (up - fu) * Su.rdp) * (s * (T(0.5) * Su.h));
-            div += fabs(xa[a]) * rh[ty][a] * (fout - fin); // zero for a zero component
-          }
-          T cq = T(0);
-#pragma unroll
-          for (int a = 0; a < 3; ++a) cq += cv[a] * q[a];
-          const T e = pre * exp_t(-c2 * invT);
-          const T g = e * (T(1) + shA * cq * (T(2) * c2 * invT - T(5)));
-          T fo[NC];
-          fo[0] = fc - A.dt * div + dtau * (g - fc);
-          A.fn[(size_t)c * A.nvp + k] = fo[0];
-          moments(cv, c2, A.w[k], fo);
-        }
-      } else {
-        general();
       }
     } else {
       general();
@@ -2193,7 +1998,6 @@ template <typename T, int D> cudaError_t tree_sweep_t(ibdvm_ctx *ctx) {
     A.stg = reinterpret_cast<const double2 *>(ctx->tree_stg);
     A.lrec = reinterpret_cast<const int4 *>(ctx->tree_lrec);
     A.sched = ctx->tree_sched;
-    for (int i = 0; i < 3; ++i) A.qb[i] = ctx->tree_qb[i];
     dim3 block(kThreadsPerCell, kCellsPerBlock);
     dim3 grid((unsigned)((ctx->ncell + kCellsPerBlock - 1) / kCellsPerBlock), (unsigned)ctx->nchunk);
     tree_sweep_kernel<T, D><<<grid, block, 0, ctx->stream>>>(A);
@@ -2539,7 +2343,7 @@ cudaError_t launch_sweep(ibdvm_ctx *ctx) {
         e = ctx->tree ? tree_sweep_t<T, D>(ctx) : sweep64_launch(ctx);
       } else {
         ctx->kernel_launches[kKSweep] += 1;
-        e = ctx->tree ? tree_sweep_t<T, D>(ctx)
+        e = ctx->tree ? tree_sweep32_launch(ctx)
             : tma     ? (D == 2 ? tma_sweep_launch(ctx) : tma3_sweep_launch(ctx))
                       : sweep_t<T, D>(ctx, 1, 1);
       }
