@@ -597,7 +597,7 @@ void upload_tree_tables(ibdvm_ctx *ctx, const std::vector<int> &glink, const std
   upload(ctx, ctx->tree_sti, sti, "upload tree stencils");
   upload(ctx, ctx->tree_stg, stg, "upload tree stencil geometry");
   upload(ctx, ctx->tree_lrec, lrec, "upload tree leaf records");
-  upload(ctx, ctx->tree_sched, tree_schedule(ctx->dim, lrec), "upload tree leaf schedule");
+  upload(ctx, ctx->tree_sched, tree_schedule(ctx->dim, lrec, ctx->precision != IBDVM_FP64, &ctx->tree_nreg), "upload tree leaf schedule");
   cfree_t(ctx->tree_far);
   if (!far.empty()) {
     ctx->tree_far = dalloc<int>(ctx, far.size(), "tree donor rows");
@@ -783,7 +783,7 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
       upload(ctx, ctx->tree_sti, sti, "upload tree stencils");
       upload(ctx, ctx->tree_stg, stg, "upload tree stencil geometry");
       upload(ctx, ctx->tree_lrec, lrec, "upload tree leaf records");
-      upload(ctx, ctx->tree_sched, tree_schedule(G.dim, lrec), "upload tree leaf schedule");
+      upload(ctx, ctx->tree_sched, tree_schedule(G.dim, lrec, ctx->precision != IBDVM_FP64, &ctx->tree_nreg), "upload tree leaf schedule");
       ctx->tree_nb_h = std::move(tnb);
     }
     ctx->kst = dalloc<int>(ctx, G.nv, "velocity positions");

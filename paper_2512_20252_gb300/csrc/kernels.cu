@@ -2342,7 +2342,8 @@ cudaError_t launch_sweep(ibdvm_ctx *ctx) {
         ctx->kernel_launches[kKSweep] += ctx->tree ? 1 : sweep64_launches(ctx);
         e = ctx->tree ? tree_sweep_t<T, D>(ctx) : sweep64_launch(ctx);
       } else {
-        ctx->kernel_launches[kKSweep] += 1;
+        // (a tree: the regular leaves and the others)
+        ctx->kernel_launches[kKSweep] += ctx->tree ? (ctx->tree_nreg > 0) + (ctx->tree_nreg < ctx->ncell) : 1;
         e = ctx->tree ? tree_sweep32_launch(ctx)
             : tma     ? (D == 2 ? tma_sweep_launch(ctx) : tma3_sweep_launch(ctx))
                       : sweep_t<T, D>(ctx, 1, 1);

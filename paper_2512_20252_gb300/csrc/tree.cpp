@@ -215,14 +215,21 @@ void build_tree_stencils(int D, const std::vector<int> &lev, const std::vector<i
 // Z order), the regular leaves (the gather-first path), then the other fluid
 // leaves (the general path), then the solid ones, so that the four leaves of
 // a block take paths of about the same length while the blocks of a window
-// share the rows they read.
-std::vector<int> tree_schedule(int D, const std::vector<int> &lrec) {
+// share the rows they read.  split (the FP32 sweep, which launches the regular
+// leaves by themselves): all regular leaves first, then the others by window.
+std::vector<int> tree_schedule(int D, const std::vector<int> &lrec, bool split, int *nreg) {
   constexpr size_t kWindow = 256;
   const size_t n = lrec.size() / 8;
+  *nreg = 0;
   std::vector<int> sched;
   sched.reserve(n);
+  if (split) {
+    for (size_t c = 0; c < n; ++c)
+      if (lrec[c * 8 + 2 * D + 1] != 0 && lrec[c * 8 + 2 * D] != 0) sched.push_back(static_cast<int>(c));
+    *nreg = static_cast<int>(sched.size());
+  }
   for (size_t w0 = 0; w0 < n; w0 += kWindow)
-    for (int cls = 0; cls < 3; ++cls)
+    for (int cls = split ? 1 : 0; cls < 3; ++cls)
       for (size_t c = w0; c < std::min(n, w0 + kWindow); ++c) {
         const bool fluid = lrec[c * 8 + 2 * D + 1] != 0, regular = lrec[c * 8 + 2 * D] != 0;
         if ((fluid && regular ? 0 : fluid ? 1 : 2) == cls) sched.push_back(static_cast<int>(c));

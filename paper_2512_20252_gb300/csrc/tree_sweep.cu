@@ -8,7 +8,7 @@
 // value, the mean of the face values over a side shared with finer leaves.
 // Organised for GB300 around vectors of 16 bytes:
 //
-//   * 64 threads take a leaf, four leaves a block; a thread takes 16 bytes of a
+//   * 64 threads take a leaf, two leaves a block; a thread takes 16 bytes of a
 //     row at a time (four velocities of an octree, the (h, b) pairs of two of a
 //     quadtree), so every gather is a 16-byte load of consecutive addresses
 //     across a warp and the faces run on packed FP32 pairs;
@@ -21,16 +21,22 @@
 //     gather-first path: the leaf, its 2 D neighbours and the D far neighbours
 //     upwind, all loads issued before any arithmetic (the upwind leaf's value
 //     and its side towards the leaf are the leaf's side value and own value);
-//   * the stencil tables are built once on the host (tree.cpp) and read into
-//     shared memory per block.
+//   * those leaves and the others are two launches, each with the registers and
+//     the shared tables that it needs.  The stencil tables are built once on the
+//     host (tree.cpp) and read into shared memory per block.
 //
-// Measured (sweep launch): octree sphere of 46,584 leaves x 20^3 velocities 2.91 ms,
-// where scalar gathers had taken 6.34; Ma 5 cylinder of 69,148 leaves x 60^2 1.63 ms
-// (1.77).  Three blocks per SM (80 registers, some spills): two 3.48 / 1.81 ms, four
-// 3.20 / 1.84.
+// What bounds it: the latency of the gathers (the stalls on them are 7 of 12 warps
+// per issue) and their L2 traffic (58% of its rate for the regular leaves).
+// Measured per step: octree sphere of 46,584 leaves x 20^3 velocities 2.85 ms (1.57
+// for the 33,050 regular leaves), where scalar gathers had taken 6.34; Ma 5 cylinder
+// of 69,148 leaves x 60^2 1.54 ms (1.77).  Both kinds of leaf in one launch, 80
+// registers: 2.91 / 1.63; blocks of four leaves, four per SM: 2.95 / 1.62; eight and
+// nine blocks of two: 3.01 / 1.62 and 3.79 / 1.85; pieces of one orthant per warp
+// from a table: 3.13 / 2.14; 32 threads per leaf, eight leaves: 3.12 / 1.83.
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 #include "ctx.h"
 #include "tma_sync.cuh"
@@ -41,7 +47,8 @@ namespace {
 using namespace dev;
 
 constexpr int kTreeThreads = 64; // threads of a leaf
-constexpr int kTreeLeaves = 4;   // leaves of a block
+constexpr int kTreeLeaves = 2;   // leaves of a block
+constexpr int kTreeBlocks = 7;   // blocks per SM (72 registers: 14 warps more than at 128 hide the gathers better)
 constexpr float kLn2 = 0.693147180559945309f;
 constexpr float kLog2e = 1.442695040888963407f;
 
@@ -56,7 +63,7 @@ struct Tree32Args {
   const int4 *__restrict__ lrec;   // [leaf][2]: leaves on the sides, regular flag, fluid flag
   const int *__restrict__ sched;
   long long ncell;
-  int nv, nvp, kloop;
+  int nv, nvp, per, nleaf; // per: velocities of a chunk; nleaf: leaves of this launch (sched)
   float dt;
   int qb[7]; // first stored position of the orthants 1 .. 2^D - 1 (bit a: component a < 0)
 };
@@ -109,42 +116,49 @@ __device__ __forceinline__ float ex2(float x) {
 __device__ __forceinline__ void acc_add(float &a, float2 v) { a += v.x + v.y; }
 __device__ __forceinline__ void acc_fma(float &a, float2 u, float2 v) { a = fmaf(u.y, v.y, fmaf(u.x, v.x, a)); }
 
-template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3) tree_sweep32_kernel(Tree32Args A) {
+template <int D, bool REG>
+__global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_sweep32_kernel(Tree32Args A) {
   constexpr int NC = (D == 2) ? 2 : 1;
   constexpr int NM = (D == 2) ? 9 : 14;
   constexpr int NF = 1 << (D - 1); // leaves at most beyond a face
   constexpr int NS = 2 * D;        // sides
   constexpr int E = tree_entries(D), EI = tree_entry_ints(D);
   constexpr int VE = 4 / NC;       // velocities of a vector
-  __shared__ float red[kTreeLeaves][2][NM];
+  constexpr int W = kTreeThreads / 32; // warps of a leaf
+  __shared__ float red[kTreeLeaves][W][NM];
   // per leaf: its own stencil along each axis, then the upwind neighbours'
   // along axis a, side sd (0: -, 1: +), neighbour j at D + (2a + sd) NF + j
   __shared__ Stencil<NF> st[kTreeLeaves][E];
   __shared__ float s_rh[kTreeLeaves][D]; // dt / h
+  // the leaf's Shakhov parameters as packed pairs: -U, -log2(e)/T, prefactor,
+  // A (1 - Pr) q, dt/tau (read again for every vector: registers are what limits
+  // the loads in flight)
+  __shared__ float2 s_c[kTreeLeaves][9];
+  __shared__ float s_T[kTreeLeaves]; // T / 2
   __shared__ int rec[kTreeLeaves][8];    // leaves on side 2a + sd (0 domain edge, 1, NF, 3 a ghost), regular, fluid
   const int tx = threadIdx.x, ty = threadIdx.y;
   const long long slot = (long long)blockIdx.x * kTreeLeaves + ty;
-  const bool active = slot < A.ncell;
+  const bool active = slot < A.nleaf;
   const long long c = active ? A.sched[slot] : 0;
   const int chunk = blockIdx.y;
+  auto row = [&](int i) -> const float * {
+    return (i >= 0) ? A.f + (size_t)i * A.nvp * NC
+           : (i == -2) ? A.finf
+           : (i <= -3) ? A.lval + (size_t)(-3 - i) * A.nvp * NC // a ghost's value for this leaf (C29)
+                       : nullptr;
+  };
   if (active && tx < E) {
-    const size_t e = (size_t)c * E + tx;
+    const int4 *I4 = A.sti + ((size_t)c * E + tx) * (EI / 4);
     int I[EI];
 #pragma unroll
     for (int q = 0; q < EI / 4; ++q) {
-      const int4 v = A.sti[e * (EI / 4) + q];
+      const int4 v = I4[q];
       I[4 * q] = v.x;
       I[4 * q + 1] = v.y;
       I[4 * q + 2] = v.z;
       I[4 * q + 3] = v.w;
     }
-    const double2 g0 = A.stg[2 * e], g1 = A.stg[2 * e + 1];
-    auto row = [&](int i) -> const float * {
-      return (i >= 0) ? A.f + (size_t)i * A.nvp * NC
-             : (i == -2) ? A.finf
-             : (i <= -3) ? A.lval + (size_t)(-3 - i) * A.nvp * NC // a ghost's value for this leaf (C29)
-                         : nullptr;
-    };
+    const double2 g0 = A.stg[2 * ((size_t)c * E + tx)], g1 = A.stg[2 * ((size_t)c * E + tx) + 1];
     Stencil<NF> S;
     S.c = row(I[0]);
 #pragma unroll
@@ -158,28 +172,27 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
     S.h = (float)g1.x;
     st[ty][tx] = S;
     if (tx < D) s_rh[ty][tx] = A.dt * (float)g1.y;
-  } else if (active && tx >= 32 && tx < 40) {
-    rec[ty][tx - 32] = reinterpret_cast<const int *>(A.lrec)[(size_t)c * 8 + tx - 32];
+  }
+  if (active && tx >= 40 && tx < 48) rec[ty][tx - 40] = reinterpret_cast<const int *>(A.lrec)[(size_t)c * 8 + tx - 40];
+  if (active && tx == 63) {
+    const float *M = A.mac + c * kMac;
+    const float sh = M[kShA]; // the Shakhov factor A (1 - Pr) folded into the heat flux
+    const float v[9] = {-M[kU0], -M[kU0 + 1], -M[kU0 + 2], -M[kInvT] * kLog2e, M[kPre],
+                        sh * M[kQ0], sh * M[kQ0 + 1], sh * M[kQ0 + 2], M[kDtTau]};
+#pragma unroll
+    for (int i = 0; i < 9; ++i) s_c[ty][i] = dup(v[i]);
+    s_T[ty] = M[kHalfT];
   }
   __syncthreads();
   float acc[NM];
 #pragma unroll
   for (int m = 0; m < NM; ++m) acc[m] = 0.f;
   if (active) {
-    const float4 *M4 = reinterpret_cast<const float4 *>(A.mac + c * kMac);
-    const float4 m0 = M4[0], m1 = M4[1], m2 = M4[2];
-    const float2 mU[3] = {dup(-m0.y), dup(-m0.z), dup(-m0.w)};
-    const float2 pre2 = dup(m0.x), nl2 = dup(-m1.x * kLog2e);
-    const float halfT = m1.y, T = 2.f * m1.y;
-    const float2 q[3] = {dup(m1.z * m1.w), dup(m1.z * m2.x), dup(m1.z * m2.y)}; // the Shakhov factor folded in
-    const float dtau = m2.z;
-    float rh[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) rh[a] = s_rh[ty][a];
+    const float2 *C = s_c[ty]; // -U_x, -U_y, -U_z, -log2(e) / T, prefactor, q_x, q_y, q_z, dt / tau
+    const float halfT = s_T[ty];
     const float *own = A.f + (size_t)c * A.nvp * NC;
     float *dst = A.fn + (size_t)c * A.nvp * NC;
-    const int kbeg = chunk * A.kloop * kTreeThreads, kend = min(A.nv, kbeg + A.kloop * kTreeThreads);
-    const bool fluid = rec[ty][NS + 1] != 0, fast = rec[ty][NS] != 0;
+    const int k0 = chunk * A.per, k1 = min(A.nv, k0 + A.per); // the velocities of this chunk
     auto orthant = [&](int k) {
       int o = 0;
 #pragma unroll
@@ -211,14 +224,14 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
         v.w[0] = __ldg(reinterpret_cast<const float2 *>(A.w + k));
       }
     };
-    // -(|a| face difference) of axis a added to n: the coefficients of the vector's elements
+    // the flux difference d of axis a added to n
     auto flux = [&](const Vel &v, int a, V4 d, V4 n) -> V4 {
+      const float h = s_rh[ty][a];
       if constexpr (D == 3) {
-        const float2 r = dup(rh[a]);
-        return fma4(__fmul2_rn(make_float2(fabsf(v.x[a][0].x), fabsf(v.x[a][0].y)), r),
-                    __fmul2_rn(make_float2(fabsf(v.x[a][NP - 1].x), fabsf(v.x[a][NP - 1].y)), r), d, n);
+        return fma4(__fmul2_rn(make_float2(fabsf(v.x[a][0].x), fabsf(v.x[a][0].y)), dup(h)),
+                    __fmul2_rn(make_float2(fabsf(v.x[a][NP - 1].x), fabsf(v.x[a][NP - 1].y)), dup(h)), d, n);
       } else {
-        return fma4(dup(fabsf(v.x[a][0].x) * rh[a]), dup(fabsf(v.x[a][0].y) * rh[a]), d, n);
+        return fma4(dup(fabsf(v.x[a][0].x) * h), dup(fabsf(v.x[a][0].y) * h), d, n);
       }
     };
     // relaxation towards the Shakhov equilibrium (Sec. 4 reduced forms in 2D, g^S in 3D)
@@ -227,16 +240,16 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
         float2 c2, cq;
-        const float2 cx = __fadd2_rn(v.x[0][p], mU[0]), cy = __fadd2_rn(v.x[1][p], mU[1]);
+        const float2 cx = __fadd2_rn(v.x[0][p], C[0]), cy = __fadd2_rn(v.x[1][p], C[1]);
         c2 = __ffma2_rn(cx, cx, __fmul2_rn(cy, cy));
-        cq = __ffma2_rn(cx, q[0], __fmul2_rn(cy, q[1]));
+        cq = __ffma2_rn(cx, C[5], __fmul2_rn(cy, C[6]));
         if constexpr (D == 3) {
-          const float2 cz = __fadd2_rn(v.x[D - 1][p], mU[2]);
+          const float2 cz = __fadd2_rn(v.x[D - 1][p], C[2]);
           c2 = __ffma2_rn(cz, cz, c2);
-          cq = __ffma2_rn(cz, q[2], cq);
+          cq = __ffma2_rn(cz, C[7], cq);
         }
-        const float2 tn = __fmul2_rn(c2, nl2); // -c^2 / T log2(e)
-        const float2 e = __fmul2_rn(pre2, make_float2(ex2(tn.x), ex2(tn.y)));
+        const float2 tn = __fmul2_rn(c2, C[3]); // -c^2 / T log2(e)
+        const float2 e = __fmul2_rn(C[4], make_float2(ex2(tn.x), ex2(tn.y)));
         const float2 mm = __fmul2_rn(e, cq);
         if constexpr (D == 3) {
           const float2 g = __ffma2_rn(mm, __ffma2_rn(tn, dup(-2.f * kLn2), dup(-5.f)), e);
@@ -244,12 +257,12 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
           else eq.h = g;
         } else {
           const float2 H = __ffma2_rn(mm, __ffma2_rn(tn, dup(-2.f * kLn2), dup(-4.f)), e);
-          const float2 B = __ffma2_rn(mm, __ffma2_rn(tn, dup(-T * kLn2), dup(-T)), __fmul2_rn(dup(halfT), e));
+          const float2 B = __ffma2_rn(mm, __ffma2_rn(tn, dup(-2.f * halfT * kLn2), dup(-2.f * halfT)), __fmul2_rn(dup(halfT), e));
           eq.l = make_float2(H.x, B.x);
           eq.h = make_float2(H.y, B.y);
         }
       }
-      const float2 dt2 = dup(dtau);
+      const float2 dt2 = C[8];
       return fma4(dt2, dt2, eq - f, f);
     };
     // the moment sums of a vector of values n about the bulk velocity
@@ -257,8 +270,8 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
       if constexpr (D == 3) {
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-          const float2 cx = __fadd2_rn(v.x[0][p], mU[0]), cy = __fadd2_rn(v.x[1][p], mU[1]);
-          const float2 cz = __fadd2_rn(v.x[D - 1][p], mU[2]);
+          const float2 cx = __fadd2_rn(v.x[0][p], C[0]), cy = __fadd2_rn(v.x[1][p], C[1]);
+          const float2 cz = __fadd2_rn(v.x[D - 1][p], C[2]);
           const float2 wf = __fmul2_rn(v.w[p], p == 0 ? n.l : n.h);
           const float2 xw = __fmul2_rn(cx, wf), yw = __fmul2_rn(cy, wf), zw = __fmul2_rn(cz, wf);
           const float2 c2 = __ffma2_rn(cx, cx, __ffma2_rn(cy, cy, __fmul2_rn(cz, cz)));
@@ -278,7 +291,7 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
           acc_fma(acc[13], cz, e2);
         }
       } else {
-        const float2 cx = __fadd2_rn(v.x[0][0], mU[0]), cy = __fadd2_rn(v.x[1][0], mU[1]);
+        const float2 cx = __fadd2_rn(v.x[0][0], C[0]), cy = __fadd2_rn(v.x[1][0], C[1]);
         const float2 c2 = __ffma2_rn(cx, cx, __fmul2_rn(cy, cy));
         const float2 wh = __fmul2_rn(v.w[0], make_float2(n.l.x, n.h.x));
         const float2 e2 = __ffma2_rn(c2, wh, __fmul2_rn(v.w[0], make_float2(n.l.y, n.h.y)));
@@ -295,7 +308,8 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
       }
     };
     // f^{n+1} of a vector whose velocities lie in orthant o
-    auto regular = [&](int o, int e, const Vel &v) -> V4 {
+    auto regular = [&](int o, int k, const Vel &v) -> V4 {
+      const int e = k * NC;
       const V4 f = ld4(own, e);
       V4 up[D], dn[D], far[D];
 #pragma unroll
@@ -309,9 +323,9 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
       V4 n = relax(v, f);
 #pragma unroll
       for (int a = 0; a < D; ++a) {
+        // equal spacing but towards the far leaf, which may be coarser
         const int sd = (o >> a) & 1;
         const Stencil<NF> &Su = st[ty][D + (2 * a + sd) * NF];
-        // equal spacing but towards the far leaf, which may be coarser
         const V4 b = f - up[a];
         const V4 out = f + vl4(b, dn[a] - f);
         const V4 in = up[a] + vl4((up[a] - far[a]) * ((sd ? Su.rdp : Su.rdm) * Su.h), b);
@@ -319,7 +333,8 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
       }
       return n;
     };
-    auto general = [&](int o, int e, const Vel &v) -> V4 {
+    auto general = [&](int o, int k, const Vel &v) -> V4 {
+      const int e = k * NC;
       const V4 f = ld4(own, e);
       V4 n = relax(v, f);
 #pragma unroll 1
@@ -351,7 +366,7 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
           }
         }
         const V4 d = in - out;
-        // (a is a run-time index here: the coefficients by selection)
+        // (a is a run-time index here: the components by selection)
         if (a == 0) n = flux(v, 0, d, n);
         else if (a == 1) n = flux(v, 1, d, n);
         else n = flux(v, D - 1, d, n);
@@ -359,38 +374,45 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
       return n;
     };
     auto sweep = [&](auto update) {
-      for (int k = kbeg + VE * tx; k < kend; k += VE * kTreeThreads) {
+      for (int k = k0 + VE * tx; k < k1; k += VE * kTreeThreads) {
+        asm volatile("" ::: "memory"); // the shared parameters are not kept in registers across vectors
         Vel v;
         velocities(k, v);
-        const int e = k * NC, o0 = orthant(k), k1 = min(k + VE, A.nv) - 1;
-        V4 n = update(o0, e, v);
-        if (orthant(k1) != o0 || k + VE > A.nv) {
-          // orthants meet in this vector, or padding ends it (which keeps zeros)
-          float *x = reinterpret_cast<float *>(&n);
-          for (int o = o0 + 1; o <= orthant(k1); ++o) {
-            const V4 t = update(o, e, v);
-            const float *y = reinterpret_cast<const float *>(&t);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              if (orthant(k + i / NC) == o) x[i] = y[i];
+        int o = orthant(k);
+        const int o1 = orthant(min(k + VE, A.nv) - 1);
+        // a straddling vector: orthants meet in it, or padding ends it (which keeps zeros)
+        const bool meet = o1 != o || k + VE > A.nv;
+        V4 n{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll 1
+        for (;; ++o) {
+          const V4 t = update(o, k, v);
+          if (!meet) {
+            n = t;
+            break;
           }
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (k + i / NC >= A.nv) x[i] = 0.f;
+          auto take = [&](float &x, float y, int i) {
+            const int ki = k + i / NC;
+            if (ki < A.nv && orthant(ki) == o) x = y;
+          };
+          take(n.l.x, t.l.x, 0);
+          take(n.l.y, t.l.y, 1);
+          take(n.h.x, t.h.x, 2);
+          take(n.h.y, t.h.y, 3);
+          if (o >= o1) break;
         }
-        *reinterpret_cast<float4 *>(dst + e) = make_float4(n.l.x, n.l.y, n.h.x, n.h.y);
+        *reinterpret_cast<float4 *>(dst + k * NC) = make_float4(n.l.x, n.l.y, n.h.x, n.h.y);
         moments(v, n);
       }
     };
-    if (!fluid) {
+    if constexpr (REG) {
+      sweep(regular);
+    } else if (rec[ty][NS + 1] == 0) {
       // a solid leaf (C29): not updated; the moments of its stored values
-      for (int k = kbeg + VE * tx; k < kend; k += VE * kTreeThreads) {
+      for (int k = k0 + VE * tx; k < k1; k += VE * kTreeThreads) {
         Vel v;
         velocities(k, v);
         moments(v, ld4(own, k * NC));
       }
-    } else if (fast) {
-      sweep(regular);
     } else {
       sweep(general);
     }
@@ -406,7 +428,12 @@ template <int D> __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, 3)
   }
   __syncthreads();
   if (active && tx < NM)
-    A.part[((size_t)chunk * NM + tx) * A.ncell + c] = (double)red[ty][0][tx] + (double)red[ty][1][tx];
+  {
+    double v = (double)red[ty][0][tx];
+#pragma unroll
+    for (int w = 1; w < W; ++w) v += (double)red[ty][w][tx];
+    A.part[((size_t)chunk * NM + tx) * A.ncell + c] = v;
+  }
 }
 
 } // namespace
@@ -424,20 +451,27 @@ cudaError_t tree_sweep32_launch(ibdvm_ctx *ctx) {
   A.sti = reinterpret_cast<const int4 *>(ctx->tree_sti);
   A.stg = reinterpret_cast<const double2 *>(ctx->tree_stg);
   A.lrec = reinterpret_cast<const int4 *>(ctx->tree_lrec);
-  A.sched = ctx->tree_sched;
   A.ncell = ctx->ncell;
   A.nv = ctx->nv;
   A.nvp = ctx->nvp;
-  A.kloop = ctx->kloop;
   A.dt = (float)ctx->geom.dt;
+  A.per = ctx->kloop * 64;
   for (int i = 0; i < 7; ++i) A.qb[i] = ctx->tree_qb[i];
   const dim3 block(kTreeThreads, kTreeLeaves);
-  const dim3 grid((unsigned)((ctx->ncell + kTreeLeaves - 1) / kTreeLeaves), (unsigned)ctx->nchunk);
-  if (ctx->dim == 2)
-    tree_sweep32_kernel<2><<<grid, block, 0, ctx->stream>>>(A);
-  else
-    tree_sweep32_kernel<3><<<grid, block, 0, ctx->stream>>>(A);
-  return cudaGetLastError();
+  auto launch = [&](auto kernel, int first, int n) -> cudaError_t {
+    if (n == 0) return cudaSuccess;
+    A.sched = ctx->tree_sched + first;
+    A.nleaf = n;
+    const dim3 grid((unsigned)((n + kTreeLeaves - 1) / kTreeLeaves), (unsigned)ctx->nchunk);
+    kernel<<<grid, block, 0, ctx->stream>>>(A);
+    return cudaGetLastError();
+  };
+  const int nreg = ctx->tree_nreg, nall = (int)ctx->ncell;
+  const cudaError_t e = (ctx->dim == 2) ? launch(tree_sweep32_kernel<2, true>, 0, nreg)
+                                        : launch(tree_sweep32_kernel<3, true>, 0, nreg);
+  if (e != cudaSuccess) return e;
+  return (ctx->dim == 2) ? launch(tree_sweep32_kernel<2, false>, nreg, nall - nreg)
+                         : launch(tree_sweep32_kernel<3, false>, nreg, nall - nreg);
 }
 
 } // namespace ibdvm
