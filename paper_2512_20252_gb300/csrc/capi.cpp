@@ -166,6 +166,7 @@ void free_all(ibdvm_ctx *ctx) {
   cfree_t(ctx->resblk);
   cfree_t(ctx->d_res);
   cfree_t(ctx->d_flags);
+  cfree_t(ctx->d_count);
   cfree(ctx->xiT);
   cfree(ctx->wT);
   cfree(ctx->finf);
@@ -763,10 +764,12 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
     ctx->mac = dalloc<char>(ctx, static_cast<size_t>(kMac) * ctx->ncell * ctx->esize, "macroscopic state");
     for (int i = 0; i < 2; ++i) ctx->W[i] = dalloc<double>(ctx, static_cast<size_t>(NW + G.dim) * ctx->ncell, "W");
     ctx->part = dalloc<double>(ctx, static_cast<size_t>(ctx->nchunk) * NM * ctx->ncell, "moment sums");
-    ctx->nresblk = static_cast<int>((ctx->ncell + 255) / 256);
+    ctx->nresblk = static_cast<int>((ctx->ncell + 63) / 64); // blocks of 64 cells or more
     ctx->resblk = dalloc<double>(ctx, static_cast<size_t>(ctx->nresblk) * 2 * NW, "residual sums");
     ctx->d_res = dalloc<double>(ctx, 1, "residual");
     ctx->d_flags = dalloc<int>(ctx, 1, "flags");
+    ctx->d_count = dalloc<int>(ctx, 1, "finalize counter");
+    check(ctx, cudaMemsetAsync(ctx->d_count, 0, sizeof(int), ctx->stream), "clear finalize counter");
     ctx->d_forces = dalloc<double>(ctx, 4, "forces");
     ctx->d_step_forces = dalloc<double>(ctx, 4, "step forces");
     check(ctx, cudaMemsetAsync(ctx->d_step_forces, 0, 4 * sizeof(double), ctx->stream), "clear");

@@ -78,6 +78,7 @@ struct ibdvm_ctx {
   double *resblk = nullptr;  // residual partial sums per block
   int nresblk = 0;
   double *d_res = nullptr;   // residual scalar
+  int *d_count = nullptr;    // blocks of a finalize launch done (zero between launches)
   int *d_flags = nullptr;
   // velocity tables, indexed by the stored position of a velocity
   void *xiT = nullptr, *wT = nullptr, *finf = nullptr;

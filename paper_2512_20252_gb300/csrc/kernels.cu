@@ -853,14 +853,63 @@ template <typename T, typename P = double> struct FinalArgs {
   double mu0, omega, Pr, dt;
   int nblk;         // blocks of the finalize launch (residual partial sums)
   double *res_out;  // residual of the step
+  int *count;       // blocks of the launch done (zero between launches)
   long long c0, c1; // the cells [c0, c1) of this launch
 };
+
+// Cells (threads) of a finalize block.  The kernel is a chain of FP64 arithmetic
+// per cell (FP64 storage: a pow and a dozen divisions), so a small grid wants
+// many small blocks; the last block adds the residual sums.  Before, with blocks
+// of 256 and a kernel for the residual / now: 48^2 cells in FP64 47 / 27 us, 128^2 52 / 36,
+// octree of 46,584 leaves 51 / 35; FP32, 185 x 171 cells 35 / 31, 512^2 115 / 101, the
+// 64^3 sphere 250 / 263 (blocks of 128: 340).  Kept out: four chunks' loads at a time
+// (64^3: 466 us), several threads per cell over the chunks (64^3: 373 us; octree 64).
+template <typename T, typename P> constexpr int final_threads() {
+  return sizeof(T) == 8 ? 64 : sizeof(P) == 8 ? 128 : 256;
+}
+
+// res = max_i sqrt(sum_j dW_ij^2) / sum_j |W_ij| (Sec. 4), components with a
+// zero denominator skipped: the last block of a launch adds the blocks' sums, in
+// a fixed order
+template <int NW>
+__device__ __forceinline__ void residual_last(const double *__restrict__ resblk, int nblk, double *__restrict__ out,
+                                              double (*red)[8]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  double s[2 * NW];
+#pragma unroll
+  for (int i = 0; i < 2 * NW; ++i) s[i] = 0.0;
+  for (int b = threadIdx.x; b < nblk; b += blockDim.x)
+#pragma unroll
+    for (int i = 0; i < 2 * NW; ++i) s[i] += __ldcg(resblk + (size_t)b * 2 * NW + i);
+#pragma unroll
+  for (int i = 0; i < 2 * NW; ++i) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[i] += __shfl_down_sync(0xffffffffu, s[i], o);
+    if (lane == 0) red[i][wid] = s[i];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double r = 0.0;
+    for (int i = 0; i < NW; ++i) {
+      double num = 0.0, den = 0.0;
+      for (int w = 0; w < nw; ++w) {
+        num += red[i][w];
+        den += red[NW + i][w];
+      }
+      if (den == 0.0) continue;
+      const double v = sqrt(num) / den;
+      r = (v > r) ? v : r;
+    }
+    *out = r;
+  }
+}
 
 template <typename T, int D, typename P>
 __device__ __forceinline__ void finalize_body(const FinalArgs<T, P> &A, const int blk) {
   constexpr int NM = Dims<D>::NM;
   constexpr int NW = Dims<D>::NW;
   __shared__ double red[2 * NW][8];
+  __shared__ bool s_last;
   const long long c = A.c0 + (long long)blk * blockDim.x + threadIdx.x;
   double rnum[NW], rden[NW];
 #pragma unroll
@@ -888,11 +937,11 @@ __device__ __forceinline__ void finalize_body(const FinalArgs<T, P> &A, const in
     double V[3] = {0.0, 0.0, 0.0};
     if (A.shift)
       for (int a = 0; a < D; ++a) V[a] = (double)A.mac[c * kMac + kU0 + a];
-    const double rho = M[0];
+    const double rho = M[0], rinv = 1.0 / rho;
     double M1[3] = {0, 0, 0}, d[3] = {0, 0, 0}, d2 = 0.0, VM1 = 0.0, V2 = 0.0;
     for (int a = 0; a < D; ++a) {
       M1[a] = M[1 + a];
-      d[a] = M1[a] / rho;
+      d[a] = M1[a] * rinv;
       d2 += d[a] * d[a];
       VM1 += V[a] * M1[a];
       V2 += V[a] * V[a];
@@ -911,7 +960,7 @@ __device__ __forceinline__ void finalize_body(const FinalArgs<T, P> &A, const in
     // conservative variables (Eq. moments1) and temperature (Eq. moments2) with
     // three translational degrees of freedom: rho E = rho |U|^2 / 2 + 3/4 rho T
     const double rhoE = 0.5 * (M2 + 2.0 * VM1 + V2 * rho);
-    const double T_ = (2.0 / 3.0) * (M2 - rho * d2) / rho;
+    const double T_ = (2.0 / 3.0) * (M2 - rho * d2) * rinv;
     double q[3] = {0, 0, 0};
     for (int a = 0; a < D; ++a) {
       double s = 0.0;
@@ -984,49 +1033,23 @@ __device__ __forceinline__ void finalize_body(const FinalArgs<T, P> &A, const in
     __syncthreads();
     if (threadIdx.x < 2 * NW) {
       double s = 0.0;
-      for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[threadIdx.x][w];
       A.resblk[(size_t)blk * 2 * NW + threadIdx.x] = s;
+      __threadfence();
     }
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(A.count, 1) == A.nblk - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    residual_last<NW>(A.resblk, A.nblk, A.res_out, red);
+    if (threadIdx.x == 0) *A.count = 0;
   }
 }
 
 template <typename T, int D, typename P>
-__global__ void __launch_bounds__(256) finalize_kernel(FinalArgs<T, P> A) {
+__global__ void __launch_bounds__(final_threads<T, P>()) finalize_kernel(const __grid_constant__ FinalArgs<T, P> A) {
   finalize_body<T, D, P>(A, blockIdx.x);
-}
-
-// res = max_i sqrt(sum_j dW_ij^2) / sum_j |W_ij| (Sec. 4), components with a
-// zero denominator skipped; one block, fixed summation order
-template <int NW>
-__device__ __forceinline__ void residual_body(const double *__restrict__ resblk, int nblk, double *__restrict__ out) {
-  __shared__ double sh[256];
-  __shared__ double tot[2 * NW];
-  for (int i = 0; i < 2 * NW; ++i) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += resblk[(size_t)b * 2 * NW + i];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) tot[i] = sh[0];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int i = 0; i < NW; ++i) {
-      if (tot[NW + i] == 0.0) continue;
-      double v = sqrt(tot[i]) / tot[NW + i];
-      r = (v > r) ? v : r;
-    }
-    *out = r;
-  }
-}
-
-template <int NW>
-__global__ void residual_kernel(const double *__restrict__ resblk, int nblk, double *__restrict__ out) {
-  residual_body<NW>(resblk, nblk, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -1889,19 +1912,13 @@ __global__ void __launch_bounds__(kForceThreads) forces_grouped(const ForceArgs<
 }
 
 template <typename T, int D, typename P>
-__global__ void __launch_bounds__(256) finalize_grouped(const FinalArgs<T, P> *__restrict__ tab,
+__global__ void __launch_bounds__(final_threads<T, P>()) finalize_grouped(const FinalArgs<T, P> *__restrict__ tab,
                                                         const int *__restrict__ start, int ncase, int par) {
   __shared__ FinalArgs<T, P> sA;
   const int c = group_case(start, ncase, blockIdx.x);
   if (threadIdx.x == 0) sA = tab[2 * c + par];
   __syncthreads();
   finalize_body<T, D, P>(sA, blockIdx.x - __ldg(start + c));
-}
-
-template <typename T, int D, typename P>
-__global__ void __launch_bounds__(256) residual_grouped(const FinalArgs<T, P> *__restrict__ tab, int par) {
-  const FinalArgs<T, P> &A = tab[2 * blockIdx.x + par];
-  residual_body<Dims<D>::NW>(A.resblk, A.nblk, A.res_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -2023,7 +2040,8 @@ FinalArgs<T, P> final_args(const ibdvm_ctx *ctx, int wcur, bool shift, bool resi
   A.omega = ctx->geom.gas.omega_vhs;
   A.Pr = ctx->geom.gas.Pr;
   A.dt = ctx->geom.dt;
-  A.nblk = (int)((ctx->ncell + 255) / 256);
+  A.nblk = (int)((ctx->ncell + final_threads<T, P>() - 1) / final_threads<T, P>());
+  A.count = ctx->d_count;
   A.res_out = ctx->d_res;
   A.c0 = 0;
   A.c1 = ctx->ncell;
@@ -2038,13 +2056,8 @@ cudaError_t finalize_t(ibdvm_ctx *ctx, bool shift, bool residual, const P *part 
   else
     pp = part;
   const FinalArgs<T, P> A = final_args<T, P>(ctx, ctx->wcur, shift, residual, pp, nchunk ? nchunk : ctx->nchunk);
-  finalize_kernel<T, D, P><<<A.nblk, 256, 0, ctx->stream>>>(A);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (residual) {
-    residual_kernel<Dims<D>::NW><<<1, 256, 0, ctx->stream>>>(ctx->resblk, A.nblk, ctx->d_res);
-    e = cudaGetLastError();
-  }
+  finalize_kernel<T, D, P><<<A.nblk, final_threads<T, P>(), 0, ctx->stream>>>(A);
+  const cudaError_t e = cudaGetLastError();
   ctx->wcur = 1 - ctx->wcur;
   return e;
 }
@@ -2250,8 +2263,8 @@ cudaError_t launch_refresh_range(ibdvm_ctx *ctx, long long c0, long long c1) {
           final_args<T, double>(ctx, pass == 0 ? ctx->wcur : 1 - ctx->wcur, pass == 1, false, ctx->part, 1);
       A.c0 = c0;
       A.c1 = c1;
-      A.nblk = (int)((c1 - c0 + 255) / 256);
-      finalize_kernel<T, D, double><<<A.nblk, 256, 0, ctx->stream>>>(A);
+      A.nblk = (int)((c1 - c0 + final_threads<T, double>() - 1) / final_threads<T, double>());
+      finalize_kernel<T, D, double><<<A.nblk, final_threads<T, double>(), 0, ctx->stream>>>(A);
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
@@ -2352,7 +2365,7 @@ cudaError_t launch_sweep(ibdvm_ctx *ctx) {
     if (e != cudaSuccess) return e;
     ctx->cur = 1 - ctx->cur;
     Timed tm(ctx, kKMoments);
-    ctx->kernel_launches[kKMoments] += 2;
+    ctx->kernel_launches[kKMoments] += 1;
     if (tma) return finalize_t<T, D, float>(ctx, true, true, ctx->partf, ctx->tma_nchunk);
     return finalize_t<T, D>(ctx, true, true);
   });
@@ -2422,7 +2435,7 @@ cudaError_t group_build(const std::vector<ibdvm_ctx *> &cases, const std::vector
     gs[i + 1] = gs[i] + (ctx->nlink ? ctx->nghost : 0);
     ss[i + 1] = ss[i] + (ctx->nlink ? slope_blocks(ctx) : 0);
     t.split = std::max(t.split, ghost_split(ctx->nvp));
-    fs[i + 1] = fs[i] + static_cast<int>((ctx->ncell + 255) / 256);
+    fs[i + 1] = fs[i] + static_cast<int>((ctx->ncell + final_threads<float, float>() - 1) / final_threads<float, float>());
     for (int p = 0; p < 2; ++p) {
       g[2 * i + p] = ghost_args<float>(ctx, ctx->cur ^ p, nullptr);
       fa[2 * i + p] = force_args<float>(ctx, ctx->cur ^ p, forces + 4 * i);
@@ -2482,15 +2495,9 @@ cudaError_t group_finalize(const GroupTables &t, int par, cudaStream_t s) {
   if (t.ncase == 0) return cudaSuccess;
   const auto *tab = static_cast<const FinalArgs<float, float> *>(t.fin);
   if (t.dim == 2)
-    finalize_grouped<float, 2, float><<<t.fin_blocks, 256, 0, s>>>(tab, t.fin_start, t.ncase, par);
+    finalize_grouped<float, 2, float><<<t.fin_blocks, final_threads<float, float>(), 0, s>>>(tab, t.fin_start, t.ncase, par);
   else
-    finalize_grouped<float, 3, float><<<t.fin_blocks, 256, 0, s>>>(tab, t.fin_start, t.ncase, par);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (t.dim == 2)
-    residual_grouped<float, 2, float><<<t.ncase, 256, 0, s>>>(tab, par);
-  else
-    residual_grouped<float, 3, float><<<t.ncase, 256, 0, s>>>(tab, par);
+    finalize_grouped<float, 3, float><<<t.fin_blocks, final_threads<float, float>(), 0, s>>>(tab, t.fin_start, t.ncase, par);
   return cudaGetLastError();
 }
 
