@@ -467,7 +467,8 @@ ibdvm_status ibdvm_batch_step(ibdvm_batch *b, int nsteps, double *residuals, int
 ibdvm_status ibdvm_batch_forces(ibdvm_batch *b, double *F, double *Q, double *CD, double *CL);
 
 /* Tiling of the sweep's work items.  rows: target rows (3D: planes) per item
-   (0 = whole columns).  kpt (0, 2 or 4) is accepted and has no effect: every
+   (0 = whole columns).  Until a tiling is set or tuned rows reads 0 and the
+   items are whole columns in 3D and about 64 rows in 2D.  kpt (0, 2 or 4) is accepted and has no effect: every
    member's sweep takes the velocity chunks of its orthant layout (2D: 192,
    128 or 64 velocities; 3D: 256 or 128), and get_tiling reports the
    velocities per lane of the first member's chunk (chunk / 32; 0 without

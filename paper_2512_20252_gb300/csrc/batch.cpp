@@ -27,6 +27,7 @@ struct ibdvm_batch {
   bool dirty = true;
   int par = 0;                  // steps since the tables were built, mod 2
   int rows = 0, kpt = 0;        // tiling of the sweep's work items (kpt: kept, no effect)
+  bool tiled = false;           // a tiling was set or tuned; until then the work list sizes its items itself
   GroupTables gt;
   SweepTables st;
   double *d_res = nullptr;      // [cap] residual of each member's last step
@@ -158,7 +159,8 @@ void build(ibdvm_batch *b) {
   }
   bcheck(b, group_build(b->members, nchunk, b->d_res, b->d_flags, b->d_forces, b->gt, b->stream),
          "build the grouped launch tables");
-  bcheck(b, tma_batch_build(b->members, kpt, b->rows, b->d_flags, b->st, b->stream), "build the sweep work list");
+  bcheck(b, tma_batch_build(b->members, kpt, b->tiled ? b->rows : -1, b->d_flags, b->st, b->stream),
+         "build the sweep work list");
   // member indices may have moved: the step forces start over
   bcheck(b, cudaMemsetAsync(b->d_forces, 0, 4 * b->cap * sizeof(double), b->stream), "clear batch forces");
   std::fill(b->stepped.begin(), b->stepped.end(), 0);
@@ -446,8 +448,9 @@ ibdvm_status ibdvm_batch_set_tiling(ibdvm_batch *b, int rows, int kpt) {
     return IBDVM_E_INVAL;
   }
   b->kpt = kpt; // no effect: every member takes the chunk of its velocity layout
-  if (rows != b->rows) {
+  if (rows != b->rows || !b->tiled) {
     b->rows = rows;
+    b->tiled = true;
     b->dirty = true;
   }
   return IBDVM_OK;
@@ -484,6 +487,7 @@ ibdvm_status ibdvm_batch_tune(ibdvm_batch *b, int steps_per_trial, double *best_
   try {
     for (int r : rows_c) {
       b->rows = r;
+      b->tiled = true;
       b->dirty = true;
       build(b);
       bcheck(b, cudaMemsetAsync(b->d_flags, 0, b->members.size() * sizeof(int), b->stream), "clear flags");

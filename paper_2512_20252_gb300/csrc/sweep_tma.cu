@@ -736,6 +736,20 @@ void tma_batch_free(SweepTables &t) {
   t = SweepTables{};
 }
 
+// Rows of an item where no tiling was set.  Whole columns leave most SMs idle at
+// the end of a chunk width's launch (one per width), and from the start when the
+// members are few; an item's own start (three rows loaded before the first update)
+// costs more the shorter it is.  Sweep of a step, whole columns / 32 / 64 / 96 /
+// 128 / 192 rows: 3 members of 159^2..332^2 cells 975 / 640 / 655 / 733 / 764 / 835
+// us, 4 of 140^2..324^2 1800 / 1114 / 1116 / 1173 / 1234 / 1470, 8 of 79^2..334^2
+// 3491 / 3420 / 3317 / 3308 / 3336 / 3380, 12 of 108^2..330^2 3888 / 3717 / 3614 /
+// 3565 / 3625 / 3716, 16 of 83^2..381^2 4600 / 4730 / 4565 / 4596 / 4569 / 4619.
+// 3D keeps whole columns, whose items are many: 2 members of 33^3 and 40^3 cells
+// 2391 us whole, 2465 in 24 or 32 planes; 4 of 42^3..58^3 13368 and 13887 (32).
+constexpr int kAutoRows = 64;
+
+// rows > 0: target rows (3D: planes) of an item; 0: whole columns; < 0: no tiling
+// was set (2D: about kAutoRows rows; 3D: whole columns)
 cudaError_t tma_batch_build(const std::vector<ibdvm_ctx *> &cases, const std::vector<int> &kpt, int rows,
                             int *flags, SweepTables &t, cudaStream_t s) {
   (void)kpt; // the chunk of every member is that of its velocity layout
@@ -759,7 +773,8 @@ cudaError_t tma_batch_build(const std::vector<ibdvm_ctx *> &cases, const std::ve
     }
     // items: column strips x velocity chunks x row ranges of about `rows` rows
     const int nx = ctx->geom.n[0], ny = ctx->geom.n[1];
-    const int nrb = (rows <= 0 || rows >= ny) ? 1 : (ny + rows - 1) / rows;
+    const int nrb = (rows < 0) ? std::max(1, (ny + kAutoRows / 2) / kAutoRows)
+                               : (rows == 0 || rows >= ny) ? 1 : (ny + rows - 1) / rows;
     const int per = (ny + nrb - 1) / nrb;
     for (int x0 = 0; x0 < nx; x0 += TX)
       for (int c = 0; c < ctx->nvp / ctx->oct_kc; ++c)
