@@ -207,10 +207,13 @@ class ClockSampler:
 BATCH_KERNEL = ("sweep2d_tma_batch_kernel", "paper_2512_20252_gb300/csrc/sweep_tma.cu")
 L2_BYTES = 129 * 1000 * 1000  # GB300 L2 cache
 
-SWEEP_KERNELS = {0: ("sweep_kernel", "paper_2512_20252_gb300/csrc/kernels.cu"),
-                 1: ("sweep2d_tma_kernel", "paper_2512_20252_gb300/csrc/sweep_tma.cu"),
-                 2: ("sweep3d_tma_kernel", "paper_2512_20252_gb300/csrc/sweep3d_tma.cu"),
-                 3: ("tree_sweep_kernel", "paper_2512_20252_gb300/csrc/kernels.cu")}
+# by sweep_variant and bytes per value
+SWEEP_KERNELS = {(0, 8): ("sweep64_kernel", "paper_2512_20252_gb300/csrc/sweep64.cu"),
+                 (0, 4): ("sweep_kernel", "paper_2512_20252_gb300/csrc/kernels.cu"),
+                 (1, 4): ("sweep2d_tma_kernel", "paper_2512_20252_gb300/csrc/sweep_tma.cu"),
+                 (2, 4): ("sweep3d_tma_kernel", "paper_2512_20252_gb300/csrc/sweep3d_tma.cu"),
+                 (3, 4): ("tree_sweep32_kernel", "paper_2512_20252_gb300/csrc/tree_sweep.cu"),
+                 (3, 8): ("tree_sweep_kernel", "paper_2512_20252_gb300/csrc/kernels.cu")}
 
 
 def pinned_moments(torch, s):
@@ -220,10 +223,11 @@ def pinned_moments(torch, s):
     return W, q
 
 
-def profiled_traffic(kernel: str, source: str, pairs: int):
+def profiled_traffic(kernel: str, source: str, pairs: int, dim: int = 0):
     """DRAM bytes per launch of the dominant kernel from the committed ncu
     summary (profiles/<kernel>_*.md, measured on a smaller case and scaled by
-    the pairs processed), or None when the kernel source changed since."""
+    the pairs processed; one that states a dimension for cases of that one), or
+    None when the kernel source changed since."""
     import glob
     import hashlib
 
@@ -234,10 +238,11 @@ def profiled_traffic(kernel: str, source: str, pairs: int):
     for path in glob.glob(os.path.join(ROOT, "profiles", kernel + "_*.md")):
         fields = {}
         for line in open(path):
-            if ":" in line and line.split(":")[0] in ("traffic_bytes_per_pair", "source_sha1"):
+            if ":" in line and line.split(":")[0] in ("traffic_bytes_per_pair", "source_sha1", "dim"):
                 k, v = line.split(":", 1)
                 fields[k.strip()] = v.strip()
-        if fields.get("source_sha1") == sha and "traffic_bytes_per_pair" in fields:
+        if (fields.get("source_sha1") == sha and "traffic_bytes_per_pair" in fields
+                and fields.get("dim", str(dim)) == str(dim)):
             return float(fields["traffic_bytes_per_pair"]) * pairs
     return None
 
@@ -251,10 +256,10 @@ FP64_NOMINAL_TFLOPS = 1.25
 def profiled_fp64_flops_per_pair(dim: int):
     """FP64 operations per (cell, velocity) pair of the FP64 sweep (an FMA
     counted as two), from the committed ncu count of its executed FP64
-    instructions (profiles/sweep_kernel_fp64_*.md), or None."""
+    instructions (profiles/sweep64_kernel_*.md), or None."""
     import glob
 
-    for path in glob.glob(os.path.join(ROOT, "profiles", "sweep_kernel_fp64_*.md")):
+    for path in glob.glob(os.path.join(ROOT, "profiles", "sweep64_kernel_*.md")):
         fields = {}
         for line in open(path):
             if ":" in line and line.split(":")[0] in ("fp64_flops_per_pair", "dim"):
@@ -786,10 +791,11 @@ def measure_case(args, workload, world, rank, local, pg, with_cpu=True):
     elapsed_ms = max_over_ranks(elapsed_ms, pg)
     value = job_value(pairs, args.steps, world, elapsed_ms / 1e3)
     sweep_ms, sweep_n = kt["sweep"]
-    kname, ksrc = SWEEP_KERNELS.get(int(info.sweep_variant), SWEEP_KERNELS[0])
+    sweep_step_ms = sweep_ms / args.steps  # FP64 and tree sweeps take several launches a step
+    kname, ksrc = SWEEP_KERNELS[int(info.sweep_variant), esize]
     alg_bytes = pairs * ncomp * esize * 2  # read f^n, write f^{n+1}
     peak, peak_kind = peaks()
-    achieved = alg_bytes / (sweep_ms / sweep_n / 1e3) / 1e9 if sweep_n else None
+    achieved = alg_bytes / (sweep_step_ms / 1e3) / 1e9 if sweep_n else None
     launches = sum(n for _, n in kt.values())
     F, Q, CD, CL = solver.step_forces()
 
@@ -820,9 +826,9 @@ def measure_case(args, workload, world, rank, local, pg, with_cpu=True):
         cpu = cpu_baseline(cpu_sample_case(case), args.cpu_sample_seconds, "the workload's gas, body and velocity grid")
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None,
-                "traffic": profiled_traffic(kname, ksrc, pairs),
+                "traffic": profiled_traffic(kname, ksrc, pairs, int(info.dim)),
                 "kernel": kname, "peak_kind": peak_kind,
-                "alg_bytes_per_launch": alg_bytes, "avg_launch_ms": sweep_ms / max(sweep_n, 1)}
+                "alg_bytes_per_launch": alg_bytes, "avg_launch_ms": sweep_step_ms}
     fpp = (profiled_fp64_flops_per_pair(int(info.dim))
            if args.precision == "fp64" and not case.get("tree") else None)
     if fpp and sweep_n:
@@ -832,13 +838,13 @@ def measure_case(args, workload, world, rank, local, pg, with_cpu=True):
         sampler.start()
         peak64, peak_ms = ibdvm.fp64_fma_rate(20000, stream.cuda_stream)
         peak_clocks = sampler.stop()
-        tf = fpp * pairs / (sweep_ms / sweep_n / 1e3) / 1e12
+        tf = fpp * pairs / (sweep_step_ms / 1e3) / 1e12
         roofline = {"bound": "alu", "achieved": tf, "peak": peak64, "unit": "TFLOP/s",
-                    "frac": tf / peak64, "traffic": profiled_traffic(kname, ksrc, pairs),
+                    "frac": tf / peak64, "traffic": profiled_traffic(kname, ksrc, pairs, int(info.dim)),
                     "kernel": kname, "peak_kind": "measured FP64 FMA rate (ibdvm_fp64_fma_rate)",
                     "peak_clocks": peak_clocks, "peak_ms": peak_ms, "nominal_fp64_tflops": FP64_NOMINAL_TFLOPS,
                     "fp64_flops_per_pair": fpp,
-                    "hbm_achieved_gbs": achieved, "avg_launch_ms": sweep_ms / max(sweep_n, 1)}
+                    "hbm_achieved_gbs": achieved, "avg_launch_ms": sweep_step_ms}
     line = None
     if rank == 0:
         line = {

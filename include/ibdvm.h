@@ -157,9 +157,9 @@ typedef struct {
   int precision;
   long long steps_done;
   size_t device_bytes;
-  int sweep_variant; /* 0: plain sweep (kernels.cu), 1: TMA-staged 2D FP32 sweep (sweep_tma.cu),
-                        2: TMA-staged 3D FP32 sweep (sweep3d_tma.cu), 3: the sweep of a
-                        tree-refined grid (kernels.cu) */
+  int sweep_variant; /* 0: FP64 sweep (sweep64.cu; FP32 without TMA: kernels.cu), 1: TMA-staged 2D
+                        FP32 sweep (sweep_tma.cu), 2: TMA-staged 3D FP32 sweep (sweep3d_tma.cu),
+                        3: the sweep of a tree-refined grid (FP32 tree_sweep.cu, FP64 kernels.cu) */
 } ibdvm_info;
 
 /* Creates a context: the uniform Cartesian grid and the discrete velocity
@@ -416,14 +416,15 @@ const char *ibdvm_status_string(ibdvm_status s);
  * solves one case at a time; batching changes no arithmetic.  A member's
  * step is the one ibdvm_step takes (the same kernel bodies), launched for all
  * members at once:
- *   - one grouped ghost-band launch over every member's links (Sec. 3.2);
- *   - one grouped force launch, plus one block per member for the totals;
+ *   - grouped ghost-band launches over every member's surface entries and ghost
+ *     cells (Sec. 3.2);
+ *   - one grouped force launch, totals included;
  *   - one persistent transport / relaxation / moment sweep (Sec. 2.2, Sec. 4)
  *     over a packed work list of items, largest first, which the blocks take
  *     from a device counter: (member, 8-column strip, velocity chunk, row
  *     range) in 2D, (member, 4 x 4 column tile, 128-velocity chunk, plane
  *     range) in 3D;
- *   - one grouped finalize launch, plus one block per member for its residual.
+ *   - one grouped finalize launch, residuals included.
  * Pairs of steps replay captured CUDA graphs.
  *
  * Members are contexts in FP32 storage (IBDVM_MIXED) with the TMA sweep

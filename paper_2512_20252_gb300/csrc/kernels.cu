@@ -1,21 +1,25 @@
 // kernels.cu -- CUDA kernels (sm_103a) of one forward-Euler step of the
 // ghost-cell immersed-boundary discrete velocity method (arXiv 2512.20252).
 //
-//   ghost_band_kernel   Sec. 3.2.1-3.2.3: per link, the upwind-weighted compact
-//                       interpolation f_gc (Eqs. extrapolation 1, upwind), the
+//   surface_slopes_kernel  the FP64 slopes of every surface entry, which the ghost
+//                       cells beside it share.
+//   ghost_band_kernel   Sec. 3.2.1-3.2.3: per ghost cell, the upwind-weighted compact
+//                       interpolation f_gc (Eqs. extrapolation 1, upwind); per link, the
 //                       shifted point (Eqs. sp, fsp), the incident distribution
 //                       at the intersect point (Eq. fw), the wall density from
 //                       zero normal mass flux with the cut-cell split (Eq. rhowc,
-//                       FP64 block reduction), the cut-cell blend (Eq. fwc) and
+//                       FP64 sums over a cluster of blocks), the cut-cell blend (Eq. fwc) and
 //                       the ghost value (Eq. extrapolation 2).
-//   sweep_kernel        Sec. 2.2 and Sec. 4: per (cell, velocity), van Leer
-//                       limited upwind face values (Eqs. reconstruction,
-//                       limiter), flux divergence, Shakhov relaxation with the
-//                       reduced equilibria, forward Euler, and the velocity
-//                       moments of the new state reduced per cell.
-//   finalize_kernel     moments -> W, T, q, tau per cell; residual partial sums
-//                       (Sec. 4, FP64).
-//   forces kernels      momentum and energy through the donor-ghost faces (FP64).
+//   domain_wall_kernel  the halo values of diffuse domain walls.
+//   tree_sweep_kernel   the sweep of tree-refined grids in FP64 (FP32: tree_sweep.cu).
+//   sweep_kernel        Sec. 2.2 and Sec. 4 on uniform grids in FP32 where the TMA
+//                       sweeps (sweep_tma.cu, sweep3d_tma.cu) are not available: per
+//                       (cell, velocity), van Leer limited upwind face values (Eqs.
+//                       reconstruction, limiter), flux divergence, Shakhov relaxation
+//                       with the reduced equilibria, forward Euler, and the velocity
+//                       moments of the new state reduced per cell (FP64: sweep64.cu).
+//   finalize_kernel     moments -> W, T, q, tau per cell; the residual (Sec. 4, FP64).
+//   forces_kernel       momentum and energy through the donor-ghost faces (FP64).
 //
 // Storage type T is double (FP64 path) or float (mixed path: FP32 f, FP32
 // transport and relaxation with compensated FP32 moment sums; FP64 wall

@@ -34,7 +34,7 @@
 //     the groups the block takes.
 //
 // Measured per step, tables included, on a state with slopes everywhere: 128^2
-// cells x 40^2 velocities between walls 3.11 ms (the sweep that formed every
+// cells x 40^2 velocities between walls 3.02 ms (the sweep that formed every
 // face twice and divided took 9.55), 24^3 cells x 12^3 velocities 2.44 ms (7.48),
 // 48^2 x 24^2 0.19 ms (0.54).  The FP64 pipe is busy 86% of the time in 2D and
 // 79% in 3D, at 58 and 50 FP64 instructions per pair.  Kept out: three blocks per
@@ -631,7 +631,7 @@ void sweep64_groups(const Geom &G, std::vector<int> &out) {
   // which hold the opposite velocities: the sums of odd moments stay small as
   // they grow, and so do their roundings (heat flux of the 128^2 lid-driven
   // cavity against 64-bit tensors: 1.0e-13 relative with one list after the
-  // other, ERRNOW in turn)
+  // other, 6.9e-14 in turn)
   const size_t nb[2] = {list[0].size() / W64, list[1].size() / W64};
   for (size_t b = 0; b < std::max(nb[0], nb[1]); ++b) {
     if (b < nb[0]) gs.insert(gs.end(), list[0].begin() + b * W64, list[0].begin() + (b + 1) * W64);
