@@ -2145,14 +2145,17 @@ template <typename T, int D> cudaError_t domain_t(ibdvm_ctx *ctx) {
   return cudaGetLastError();
 }
 
-// blocks of the slope kernel
-inline int slope_blocks(const ibdvm_ctx *ctx) { return ctx->nsc * ((ctx->nvp + kSlopeVel - 1) / kSlopeVel); }
+// blocks of the slope kernel (none without upwind weighting, which reads no slopes)
+inline int slope_blocks(const ibdvm_ctx *ctx) {
+  if (ctx->nlink == 0 || (ctx->geom.gas.flags & IBDVM_NAIVE_EXTRAPOLATION)) return 0;
+  return ctx->nsc * ((ctx->nvp + kSlopeVel - 1) / kSlopeVel);
+}
 
 template <typename T, int D> cudaError_t ghost_t(ibdvm_ctx *ctx, double *dbg) {
   if (ctx->nlink == 0) return cudaSuccess;
   const GhostArgs<T> G = ghost_args<T>(ctx, ctx->cur, dbg);
-  if (!G.naive && ctx->nsc > 0) {
-    surface_slopes_kernel<T, D><<<slope_blocks(ctx), kGhostThreads, 0, ctx->stream>>>(G);
+  if (const int sb = slope_blocks(ctx)) {
+    surface_slopes_kernel<T, D><<<sb, kGhostThreads, 0, ctx->stream>>>(G);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -2300,7 +2303,7 @@ cudaError_t launch_ghost_band(ibdvm_ctx *ctx, double *dbg) {
   Timed t(ctx, kKGhost);
   // the halo values of diffuse domain walls first: the pre-ghost slopes and
   // the sweep read them
-  ctx->kernel_launches[kKGhost] += (ctx->wall_mask ? 1 : 0) + (ctx->nlink ? 2 : 0);
+  ctx->kernel_launches[kKGhost] += (ctx->wall_mask ? 1 : 0) + (slope_blocks(ctx) ? 1 : 0) + (ctx->nlink ? 1 : 0);
   return dispatch(ctx, [&](auto t, auto d) -> cudaError_t {
     using T = decltype(t);
     constexpr int D = decltype(d)::value;
@@ -2437,7 +2440,7 @@ cudaError_t group_build(const std::vector<ibdvm_ctx *> &cases, const std::vector
     const ibdvm_ctx *ctx = cases[i];
     ls[i + 1] = ls[i] + ctx->nlink;
     gs[i + 1] = gs[i] + (ctx->nlink ? ctx->nghost : 0);
-    ss[i + 1] = ss[i] + (ctx->nlink ? slope_blocks(ctx) : 0);
+    ss[i + 1] = ss[i] + slope_blocks(ctx);
     t.split = std::max(t.split, ghost_split(ctx->nvp));
     fs[i + 1] = fs[i] + static_cast<int>((ctx->ncell + final_threads<float, float>() - 1) / final_threads<float, float>());
     for (int p = 0; p < 2; ++p) {
