@@ -347,6 +347,7 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
   // millisecond beside a large state)
   const size_t band = nl * static_cast<size_t>(nvp) * ctx->ncomp * ctx->esize;
   const size_t nlv = nl * static_cast<size_t>(nvp), nsc = c_int.size() / 8;
+  const size_t f32 = (ctx->precision == IBDVM_FP64) ? 0 : 1; // the tables of FP32 storage alone
   const BodyTable tables[] = {
       {(void **)&ctx->dslot, dslot.size() * sizeof(int)},
       {(void **)&ctx->dlinks, dlinks.size() * sizeof(int)},
@@ -354,7 +355,7 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
       {(void **)&ctx->l_dbl, l_dbl.size() * sizeof(double)},
       {(void **)&ctx->l_wg, nlv * sizeof(double)},
       {(void **)&ctx->l_cn, nlv * sizeof(double)},
-      {&ctx->l_al, nlv * ctx->esize},
+      {&ctx->l_al, f32 * nlv * sizeof(float)},
       {(void **)&ctx->g_int, g_int.size() * sizeof(int)},
       {(void **)&ctx->e_int, e_int.size() * sizeof(int)},
       {(void **)&ctx->c_int, c_int.size() * sizeof(int)},
@@ -367,7 +368,7 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
       {(void **)&ctx->fpart, kForceParts * nl * sizeof(double)},
       {(void **)&ctx->fcount, sizeof(int)},
       {(void **)&ctx->gw_unit, nvp * sizeof(double)},
-      {&ctx->gw_T, nvp * ctx->esize},
+      {&ctx->gw_T, f32 * nvp * sizeof(float)},
   };
   size_t total = 0;
   for (const BodyTable &t : tables) total += (t.bytes + 255) & ~size_t(255);
@@ -409,7 +410,7 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
       gw[ctx->kst_h[k]] = norm * std::exp(-c2 / Tw);
     }
     upload(ctx, ctx->gw_unit, gw, "upload wall Maxwellian");
-    upload_typed(ctx, ctx->gw_T, gw, "upload wall Maxwellian");
+    if (f32) upload_typed(ctx, ctx->gw_T, gw, "upload wall Maxwellian");
   }
   check(ctx, launch_ghost_tables(ctx), "ghost tables kernel");
   upload(ctx, ctx->ctype, ctype, "upload cell classes");

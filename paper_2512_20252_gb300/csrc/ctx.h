@@ -113,7 +113,7 @@ struct ibdvm_ctx {
   double *l_dbl = nullptr;   // [nlink][8]
   double *l_wg = nullptr;    // [nlink][nvp]
   double *l_cn = nullptr;    // [nlink][nvp] incident mass flux per unit f (ghost_tables_kernel)
-  void *l_al = nullptr;      // [nlink][nvp] incident share of a velocity's box
+  void *l_al = nullptr;      // [nlink][nvp] incident share of a velocity's box (FP32 storage)
   int *g_int = nullptr;      // [nghost][4]: first link, links, first and last + 1 surface entry
   int *e_int = nullptr;      // [nsurf] surface cell of each entry
   int *c_int = nullptr;      // [nsc][8]: cell, codes of its face neighbours
@@ -127,7 +127,7 @@ struct ibdvm_ctx {
   double *fpart = nullptr;   // force partial sums (kForceParts per link)
   int *fcount = nullptr;     // blocks of a force launch done (zero between launches)
   double *gw_unit = nullptr; // [nvp] unit-density wall Maxwellian H_w / g_w of the body's wall
-  void *gw_T = nullptr;      // the same in the storage type
+  void *gw_T = nullptr;      // the same in FP32 (FP32 storage)
   double *d_forces = nullptr; // [4]
   double *d_step_forces = nullptr; // [4] forces of the fluxes the last step applied
   // kernel timing (CUDA events around each launch class, when enabled)

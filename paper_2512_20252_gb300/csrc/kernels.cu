@@ -1071,14 +1071,14 @@ template <typename T> struct GhostArgs {
   const double *__restrict__ l_dbl; // [nlink][8]: c_sp, c_iw, c_gc, n0, n1, n2, S, sum of ws xn G_w
   const double *__restrict__ l_wg;  // [nlink][nvp] incident-side measures
   const double *__restrict__ l_cn;  // [nlink][nvp]: wg xn, the incident mass flux per unit f
-  const T *__restrict__ l_al;       // [nlink][nvp]: wg / w, the incident share of a velocity's box
+  const T *__restrict__ l_al;       // [nlink][nvp], FP32 storage: wg / w, the incident share of a velocity's box
   const int *__restrict__ g_int;    // [nghost][4]: first link, links, first and last + 1 surface entry
   const int *__restrict__ e_int;    // [nsurf]: the surface cell of an entry (index into c_int)
   const int *__restrict__ c_int;    // [nsc][8]: surface cell, codes of its 6 face neighbours
   const T *__restrict__ s_T;        // [nsurf][8]: r (weights), |r|, x_j - x_g, 1 / |r|
   T *__restrict__ sig;              // [nsc][D][nvp][NC]: pre-ghost slopes of the surface cells
   const double *__restrict__ gwu;   // [nvp] unit-density wall Maxwellian
-  const T *__restrict__ gwT;        // the same in the storage type
+  const T *__restrict__ gwT;        // the same in FP32, FP32 storage
   const int *__restrict__ kst;      // [nv] stored position of each velocity (natural order)
   T *__restrict__ lval;
   T *__restrict__ fi;
@@ -1431,9 +1431,9 @@ template <typename T, int D> __device__ __forceinline__ void ghost_band_body(con
         T fi[NC], sp[NC], gv[NC];
         load_nc<T, NC>(G.fi + o, fi);
         load_nc<T, NC>(G.fsp + o, sp);
-        if (!G.dbg_fstar) {
-          // the wall distribution and the ghost value of the step in the storage
-          // type (the wall density above stays FP64; a launch that reports f*_w for
+        if (sizeof(T) == 4 && !G.dbg_fstar) {
+          // FP32 storage: the wall distribution and the ghost value of the step in
+          // FP32 (the wall density above stays FP64; a launch that reports f*_w for
           // the wall quantities takes the FP64 branch below, so that the normal
           // mass flux of f*_w vanishes to FP64 rounding)
           const T al = G.l_al[(size_t)l * G.nvp + k], Gw = G.gwT[k];
@@ -1445,6 +1445,9 @@ template <typename T, int D> __device__ __forceinline__ void ghost_band_body(con
             if (G.ghost_nonneg && gv[m] < T(0)) gv[m] = T(0); // optional nonnegative ghost values
           }
         } else {
+          // the reflected share from the measures' own difference: one minus a
+          // rounded incident share would leave 1e-16 of the wall's Maxwellian in
+          // velocities whose box is wholly incident, far above a cold gas's tail
           const double wk = G.wD[k], wg = G.l_wg[(size_t)l * G.nvp + k], ws = wk - wg, Gw = G.gwu[k];
 #pragma unroll
           for (int m = 0; m < NC; ++m) {
@@ -1455,7 +1458,7 @@ template <typename T, int D> __device__ __forceinline__ void ghost_band_body(con
             double v = spv + c_gc * (fstar - spv);
             if (G.ghost_nonneg && v < 0.0) v = 0.0;
             gv[m] = (T)v;
-            G.dbg_fstar[o + m] = fstar;
+            if (G.dbg_fstar) G.dbg_fstar[o + m] = fstar;
           }
         }
         store_nc<T, NC>(G.lval + o, gv);
@@ -1465,8 +1468,8 @@ template <typename T, int D> __device__ __forceinline__ void ghost_band_body(con
 }
 
 // The link tables that depend on the geometry and the wall only: per link and
-// velocity the incident mass flux per unit f and the incident share of the
-// velocity's box, per link the reflected mass flux per unit wall density
+// velocity the incident mass flux per unit f and (FP32 storage) the incident share
+// of the velocity's box, per link the reflected mass flux per unit wall density
 // (FP64; one block per link, when a body is set).
 template <typename T, int D>
 __global__ void __launch_bounds__(256) ghost_tables_kernel(GhostArgs<T> G, double *l_dbl, double *l_cn, T *l_al) {
@@ -1480,7 +1483,7 @@ __global__ void __launch_bounds__(256) ghost_tables_kernel(GhostArgs<T> G, doubl
     for (int a = 0; a < D; ++a) xn += G.xiD[a * G.nvp + k] * ld[3 + a];
     const double w = G.wD[k], wg = G.l_wg[o];
     l_cn[o] = wg * xn;
-    l_al[o] = (w > 0.0) ? (T)(wg * G.rwD[k]) : T(1);
+    if (sizeof(T) == 4) l_al[o] = (w > 0.0) ? (T)(wg * G.rwD[k]) : T(1);
     Dsum += (w - wg) * xn * G.gwu[k];
   }
   Dsum = block_sum<256>(Dsum, sh);
