@@ -864,10 +864,11 @@ template <typename T, typename P = double> struct FinalArgs {
 // Cells (threads) of a finalize block.  The kernel is a chain of FP64 arithmetic
 // per cell (FP64 storage: a pow and a dozen divisions), so a small grid wants
 // many small blocks; the last block adds the residual sums.  Before, with blocks
-// of 256 and a kernel for the residual / now: 48^2 cells in FP64 47 / 27 us, 128^2 52 / 36,
-// octree of 46,584 leaves 51 / 35; FP32, 185 x 171 cells 35 / 31, 512^2 115 / 101, the
-// 64^3 sphere 250 / 263 (blocks of 128: 340).  Kept out: four chunks' loads at a time
-// (64^3: 466 us), several threads per cell over the chunks (64^3: 373 us; octree 64).
+// of 256 and a kernel for the residual / now: 48^2 cells in FP64 39 / 27 us, 128^2 39 / 35,
+// octree of 46,584 leaves 52 / 37; FP32, 185 x 171 cells 35 / 31, 512^2 115 / 111, the
+// 64^3 sphere 249 / 245 (with products with 1 / rho for the divisions, which are less
+// exact, 262, and 101 at 512^2).  Kept out: four chunks' loads at a time (64^3: 466 us),
+// several threads per cell over the chunks (64^3: 373 us; octree 64).
 template <typename T, typename P> constexpr int final_threads() {
   return sizeof(T) == 8 ? 64 : sizeof(P) == 8 ? 128 : 256;
 }
@@ -941,11 +942,11 @@ __device__ __forceinline__ void finalize_body(const FinalArgs<T, P> &A, const in
     double V[3] = {0.0, 0.0, 0.0};
     if (A.shift)
       for (int a = 0; a < D; ++a) V[a] = (double)A.mac[c * kMac + kU0 + a];
-    const double rho = M[0], rinv = 1.0 / rho;
+    const double rho = M[0];
     double M1[3] = {0, 0, 0}, d[3] = {0, 0, 0}, d2 = 0.0, VM1 = 0.0, V2 = 0.0;
     for (int a = 0; a < D; ++a) {
       M1[a] = M[1 + a];
-      d[a] = M1[a] * rinv;
+      d[a] = M1[a] / rho; // a division: a product with 1 / rho is not exact where the quotient is
       d2 += d[a] * d[a];
       VM1 += V[a] * M1[a];
       V2 += V[a] * V[a];
@@ -964,7 +965,7 @@ __device__ __forceinline__ void finalize_body(const FinalArgs<T, P> &A, const in
     // conservative variables (Eq. moments1) and temperature (Eq. moments2) with
     // three translational degrees of freedom: rho E = rho |U|^2 / 2 + 3/4 rho T
     const double rhoE = 0.5 * (M2 + 2.0 * VM1 + V2 * rho);
-    const double T_ = (2.0 / 3.0) * (M2 - rho * d2) * rinv;
+    const double T_ = (2.0 / 3.0) * (M2 - rho * d2) / rho;
     double q[3] = {0, 0, 0};
     for (int a = 0; a < D; ++a) {
       double s = 0.0;
