@@ -27,10 +27,10 @@
 //
 // What bounds it: the latency of the gathers (the stalls on them are 7 of 12 warps
 // per issue) and their L2 traffic (58% of its rate for the regular leaves).
-// Measured per step: octree sphere of 46,584 leaves x 20^3 velocities 2.85 ms (1.57
-// for the 33,050 regular leaves), where scalar gathers had taken 6.34; Ma 5 cylinder
-// of 69,148 leaves x 60^2 1.54 ms (1.77).  Both kinds of leaf in one launch, 80
-// registers: 2.91 / 1.63; blocks of four leaves, four per SM: 2.95 / 1.62; eight and
+// Measured per step: octree sphere of 46,584 leaves x 20^3 velocities 2.80 ms, where
+// scalar gathers had taken 6.34; Ma 5 cylinder of 69,148 leaves x 60^2 1.55 ms (1.77).
+// Before the relaxation came after the fluxes, at 2.85 / 1.54: both kinds of leaf in
+// one launch, 80 registers: 2.91 / 1.63; blocks of four leaves, four per SM: 2.95 / 1.62; eight and
 // nine blocks of two: 3.01 / 1.62 and 3.79 / 1.85; pieces of one orthant per warp
 // from a table: 3.13 / 2.14; 32 threads per leaf, eight leaves: 3.12 / 1.83.
 #include <cuda_runtime.h>
@@ -49,7 +49,6 @@ using namespace dev;
 constexpr int kTreeThreads = 64; // threads of a leaf
 constexpr int kTreeLeaves = 2;   // leaves of a block
 constexpr int kTreeBlocks = 7;   // blocks per SM (72 registers: 14 warps more than at 128 hide the gathers better)
-constexpr float kLn2 = 0.693147180559945309f;
 constexpr float kLog2e = 1.442695040888963407f;
 
 struct Tree32Args {
@@ -125,15 +124,17 @@ __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_s
   constexpr int E = tree_entries(D), EI = tree_entry_ints(D);
   constexpr int VE = 4 / NC;       // velocities of a vector
   constexpr int W = kTreeThreads / 32; // warps of a leaf
-  __shared__ float red[kTreeLeaves][W][NM];
+  constexpr int NL = 8, NR = NL * W; // lanes of a warp, partial sums of a leaf, that are added in FP64
+  __shared__ float red[kTreeLeaves][NR][NM];
   // per leaf: its own stencil along each axis, then the upwind neighbours'
   // along axis a, side sd (0: -, 1: +), neighbour j at D + (2a + sd) NF + j
   __shared__ Stencil<NF> st[kTreeLeaves][E];
   __shared__ float s_rh[kTreeLeaves][D]; // dt / h
-  // the leaf's Shakhov parameters as packed pairs: -U, -log2(e)/T, prefactor,
-  // A (1 - Pr) q, dt/tau (read again for every vector: registers are what limits
-  // the loads in flight)
-  __shared__ float2 s_c[kTreeLeaves][9];
+  // the leaf's Shakhov parameters as packed pairs: -U, the factor of c^2 in the
+  // exponent (2D, base 2: -log2(e)/T; 3D: -1/T), prefactor, q, dt/tau, the
+  // Shakhov factor, 2/T (read again for every vector: registers are what
+  // limits the loads in flight)
+  __shared__ float2 s_c[kTreeLeaves][11];
   __shared__ float s_T[kTreeLeaves]; // T / 2
   __shared__ int rec[kTreeLeaves][8];    // leaves on side 2a + sd (0 domain edge, 1, NF, 3 a ghost), regular, fluid
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -176,11 +177,11 @@ __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_s
   if (active && tx >= 40 && tx < 48) rec[ty][tx - 40] = reinterpret_cast<const int *>(A.lrec)[(size_t)c * 8 + tx - 40];
   if (active && tx == 63) {
     const float *M = A.mac + c * kMac;
-    const float sh = M[kShA]; // the Shakhov factor A (1 - Pr) folded into the heat flux
-    const float v[9] = {-M[kU0], -M[kU0 + 1], -M[kU0 + 2], -M[kInvT] * kLog2e, M[kPre],
-                        sh * M[kQ0], sh * M[kQ0 + 1], sh * M[kQ0 + 2], M[kDtTau]};
+    const float v[11] = {-M[kU0],   -M[kU0 + 1], -M[kU0 + 2], (D == 2) ? -M[kInvT] * kLog2e : -M[kInvT],
+                         M[kPre],   M[kQ0],      M[kQ0 + 1],  M[kQ0 + 2],
+                         M[kDtTau], M[kShA],     2.f * M[kInvT]};
 #pragma unroll
-    for (int i = 0; i < 9; ++i) s_c[ty][i] = dup(v[i]);
+    for (int i = 0; i < 11; ++i) s_c[ty][i] = dup(v[i]);
     s_T[ty] = M[kHalfT];
   }
   __syncthreads();
@@ -188,7 +189,8 @@ __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_s
 #pragma unroll
   for (int m = 0; m < NM; ++m) acc[m] = 0.f;
   if (active) {
-    const float2 *C = s_c[ty]; // -U_x, -U_y, -U_z, -log2(e) / T, prefactor, q_x, q_y, q_z, dt / tau
+    // -U_x, -U_y, -U_z, exponent, prefactor, q_x, q_y, q_z, dt / tau, Shakhov factor, 2 / T
+    const float2 *C = s_c[ty];
     const float halfT = s_T[ty];
     const float *own = A.f + (size_t)c * A.nvp * NC;
     float *dst = A.fn + (size_t)c * A.nvp * NC;
@@ -234,8 +236,11 @@ __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_s
         return fma4(dup(fabsf(v.x[a][0].x) * h), dup(fabsf(v.x[a][0].y) * h), d, n);
       }
     };
-    // relaxation towards the Shakhov equilibrium (Sec. 4 reduced forms in 2D, g^S in 3D)
-    auto relax = [&](const Vel &v, V4 f) -> V4 {
+    // f^{n+1} of the fluxes' increment n: relaxation towards the Shakhov equilibrium
+    // (Sec. 4 reduced forms in 2D, g^S in 3D) joins the increment and f comes last,
+    // so that f^{n+1} is rounded once at its own size.  After the fluxes: the
+    // exponentials first cost 3 and 5% (octree, cylinder)
+    auto relax = [&](const Vel &v, V4 f, V4 n) -> V4 {
       V4 eq;
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
@@ -248,22 +253,23 @@ __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_s
           c2 = __ffma2_rn(cz, cz, c2);
           cq = __ffma2_rn(cz, C[7], cq);
         }
-        const float2 tn = __fmul2_rn(c2, C[3]); // -c^2 / T log2(e)
-        const float2 e = __fmul2_rn(C[4], make_float2(ex2(tn.x), ex2(tn.y)));
-        const float2 mm = __fmul2_rn(e, cq);
+        const float2 tn = __fmul2_rn(c2, C[3]);
+        // 3D: expf; a base-2 exponential of the rounded product with log2(e) errs
+        // by up to c^2/T units more
+        const float2 e = __fmul2_rn(C[4], (D == 3) ? make_float2(expf(tn.x), expf(tn.y)) : make_float2(ex2(tn.x), ex2(tn.y)));
+        const float2 mm = __fmul2_rn(e, __fmul2_rn(cq, C[9]));
         if constexpr (D == 3) {
-          const float2 g = __ffma2_rn(mm, __ffma2_rn(tn, dup(-2.f * kLn2), dup(-5.f)), e);
+          const float2 g = __ffma2_rn(mm, __ffma2_rn(tn, dup(-2.f), dup(-5.f)), e);
           if (p == 0) eq.l = g;
           else eq.h = g;
         } else {
-          const float2 H = __ffma2_rn(mm, __ffma2_rn(tn, dup(-2.f * kLn2), dup(-4.f)), e);
-          const float2 B = __ffma2_rn(mm, __ffma2_rn(tn, dup(-2.f * halfT * kLn2), dup(-2.f * halfT)), __fmul2_rn(dup(halfT), e));
+          const float2 H = __ffma2_rn(mm, __ffma2_rn(c2, C[10], dup(-4.f)), e);
+          const float2 B = __fmul2_rn(dup(halfT), __ffma2_rn(mm, dup(2.f), H));
           eq.l = make_float2(H.x, B.x);
           eq.h = make_float2(H.y, B.y);
         }
       }
-      const float2 dt2 = C[8];
-      return fma4(dt2, dt2, eq - f, f);
+      return fma4(C[8], C[8], eq - f, n) + f;
     };
     // the moment sums of a vector of values n about the bulk velocity
     auto moments = [&](const Vel &v, V4 n) {
@@ -320,7 +326,7 @@ __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_s
         dn[a] = ld4(sd ? So.m[0] : So.p[0], e);
         far[a] = ld4(sd ? Su.p[0] : Su.m[0], e);
       }
-      V4 n = relax(v, f);
+      V4 n{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
       for (int a = 0; a < D; ++a) {
         // equal spacing but towards the far leaf, which may be coarser
@@ -331,12 +337,12 @@ __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_s
         const V4 in = up[a] + vl4((up[a] - far[a]) * ((sd ? Su.rdp : Su.rdm) * Su.h), b);
         n = flux(v, a, in - out, n);
       }
-      return n;
+      return relax(v, f, n);
     };
     auto general = [&](int o, int k, const Vel &v) -> V4 {
       const int e = k * NC;
       const V4 f = ld4(own, e);
-      V4 n = relax(v, f);
+      V4 n{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll 1
       for (int a = 0; a < D; ++a) {
         const int sd = (o >> a) & 1;
@@ -371,7 +377,7 @@ __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_s
         else if (a == 1) n = flux(v, 1, d, n);
         else n = flux(v, D - 1, d, n);
       }
-      return n;
+      return relax(v, f, n);
     };
     auto sweep = [&](auto update) {
       for (int k = k0 + VE * tx; k < k1; k += VE * kTreeThreads) {
@@ -416,23 +422,35 @@ __global__ void __launch_bounds__(kTreeThreads *kTreeLeaves, kTreeBlocks) tree_s
     } else {
       sweep(general);
     }
-    if constexpr (D == 3) acc[4] = acc[5] + acc[8] + acc[10]; // the sum of w c^2 f is the trace
   }
-  // the moment sums of each leaf over its 64 threads (two warps)
+  // the moment sums of each leaf over its 64 threads (two warps): FP32 down to
+  // NL lanes a warp, the largest partial sums in FP64 (in 3D the sum of w c^2 f
+  // is the trace).  Random error of the density on a 20^3-velocity octree with all
+  // sums of a warp in FP32 / with 2, 8 and 32 lanes in FP64: 3.4, 2.6, 1.8 and 1.5e-8
 #pragma unroll
   for (int m = 0; m < NM; ++m) {
+    if (D == 3 && m == 4) continue;
     float v = acc[m];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((tx & 31) == 0) red[ty][tx >> 5][m] = v;
+    for (int o = 16; o >= NL; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((tx & 31) < NL) red[ty][NL * (tx >> 5) + (tx & 31)][m] = v;
   }
   __syncthreads();
-  if (active && tx < NM)
-  {
-    double v = (double)red[ty][0][tx];
+  if (tx < 32) { // half of the partial sums in lanes m, half in 16 + m
+    const int m = min(tx & 15, NM - 1), r0 = (tx >> 4) * (NR / 2);
+    double s[NR / 2];
 #pragma unroll
-    for (int w = 1; w < W; ++w) v += (double)red[ty][w][tx];
-    A.part[((size_t)chunk * NM + tx) * A.ncell + c] = v;
+    for (int r = 0; r < NR / 2; ++r) s[r] = (double)red[ty][r0 + r][m];
+#pragma unroll
+    for (int n = NR / 4; n > 0; n >>= 1)
+#pragma unroll
+      for (int r = 0; r < n; ++r) s[r] += s[r + n];
+    double v = s[0] + __shfl_xor_sync(0xffffffffu, s[0], 16);
+    if constexpr (D == 3) {
+      const double t = __shfl_sync(0xffffffffu, v, 5) + __shfl_sync(0xffffffffu, v, 8) + __shfl_sync(0xffffffffu, v, 10);
+      if (tx == 4) v = t;
+    }
+    if (active && tx < NM) A.part[((size_t)chunk * NM + tx) * A.ncell + c] = v;
   }
 }
 
