@@ -864,7 +864,7 @@ template <typename T, typename P = double> struct FinalArgs {
 // Cells (threads) of a finalize block.  The kernel is a chain of FP64 arithmetic
 // per cell (FP64 storage: a pow and a dozen divisions), so a small grid wants
 // many small blocks; the last block adds the residual sums.  Before, with blocks
-// of 256 and a kernel for the residual / now: 48^2 cells in FP64 39 / 27 us, 128^2 39 / 35,
+// of 256 and a kernel for the residual / now: 48^2 cells in FP64 39 / 33 us, 128^2 39 / 43,
 // octree of 46,584 leaves 52 / 37; FP32, 185 x 171 cells 35 / 31, 512^2 115 / 111, the
 // 64^3 sphere 249 / 245 (with products with 1 / rho for the divisions, which are less
 // exact, 262, and 101 at 512^2).  Kept out: four chunks' loads at a time (64^3: 466 us),
@@ -934,9 +934,32 @@ __device__ __forceinline__ void finalize_body(const FinalArgs<T, P> &A, const in
     } else {
 #pragma unroll
       for (int m = 0; m < NM; ++m) M[m] = 0.0;
-      for (int ch = 0; ch < A.nchunk; ++ch)
+      const double *pc = A.part + c;
+      const size_t st = (size_t)NM * A.ncell;
+      if constexpr (std::is_same<T, double>::value) {
+        // FP64 storage has up to 64 chunks: four at a time in pairs, and what the
+        // additions of fours round away is kept (Kahan's sum)
+        double low[NM];
 #pragma unroll
-        for (int m = 0; m < NM; ++m) M[m] += (double)A.part[((size_t)ch * NM + m) * A.ncell + c];
+        for (int m = 0; m < NM; ++m) low[m] = 0.0;
+        for (int ch = 0; ch < A.nchunk; ch += 4, pc += 4 * st) {
+          const int n = A.nchunk - ch;
+#pragma unroll
+          for (int m = 0; m < NM; ++m) {
+            const double *p = pc + (size_t)m * A.ncell;
+            const double p1 = n > 1 ? p[st] : 0.0, p2 = n > 2 ? p[2 * st] : 0.0, p3 = n > 3 ? p[3 * st] : 0.0;
+            const double y = ((p[0] + p1) + (p2 + p3)) - low[m], t = M[m] + y;
+            low[m] = (t - M[m]) - y;
+            M[m] = t;
+          }
+        }
+#pragma unroll
+        for (int m = 0; m < NM; ++m) M[m] -= low[m];
+      } else {
+        for (int ch = 0; ch < A.nchunk; ++ch, pc += st)
+#pragma unroll
+          for (int m = 0; m < NM; ++m) M[m] += pc[(size_t)m * A.ncell];
+      }
     }
     const long long nc = A.ncell;
     double V[3] = {0.0, 0.0, 0.0};

@@ -31,13 +31,16 @@
 //     per group and row;
 //   * the four warps of a block take four groups of one march direction; their
 //     sums are added in shared memory, row by row and in a fixed order, over all
-//     the groups the block takes.
+//     the groups the block takes (a compensated sum).
 //
 // Measured per step, tables included, on a state with slopes everywhere: 128^2
-// cells x 40^2 velocities between walls 3.02 ms (the sweep that formed every
-// face twice and divided took 9.55), 24^3 cells x 12^3 velocities 2.44 ms (7.48),
-// 48^2 x 24^2 0.19 ms (0.54).  The FP64 pipe is busy 86% of the time in 2D and
-// 79% in 3D, at 58 and 50 FP64 instructions per pair.  Kept out: three blocks per
+// cells x 40^2 velocities between walls 3.16 ms (the sweep that formed every
+// face twice and divided took 9.55), 24^3 cells x 12^3 velocities 2.66 ms (7.48),
+// 48^2 x 24^2 0.195 ms (0.54).  4 to 5% of these go into roundings: f^{n+1} rounded
+// once, compensated sums, the tables' exact products (without them the rms error
+// of f against extended precision was 1.2 to 1.4 times that of the sweep that
+// divided, of the sums up to 1.7 times; now 0.7 to 0.9 and 0.8 to 1.1).  Kept out, at
+// 3.02 and 2.44 ms: three blocks per
 // SM (168 registers, spills: 4.29 ms), in 2D the upwind difference along x by
 // shuffle (3.18 ms; in 3D it pays, 2.43 against 2.65 ms), the faces of a velocity
 // as parallel chains under one vote (3.21 ms: fewer are skipped).
@@ -64,9 +67,10 @@ template <int D> struct Cfg64 {
   static constexpr int CX = (D == 2) ? 16 : 8;    // columns of a tile along x
   static constexpr int CT = (D == 2) ? 16 : 32;   // columns of a tile
   static constexpr int NH = (D == 2) ? 4 : 12;    // upwind edge values of a tile per velocity (2D: 2 rows x 2 components)
-  static constexpr int MAXROWS = (D == 2) ? 32 : 16;
+  static constexpr int MAXROWS = (D == 2) ? 32 : 12;
   static size_t smem(int rows) {
-    return (size_t)(rows * NM * CT + 2 * W64 * NM * 32 + 2 * W64 * NH * KG) * sizeof(double);
+    return (size_t)(rows * NM * CT + 2 * W64 * NM * 32 + 2 * W64 * NH * KG) * sizeof(double) +
+           (size_t)rows * NM * CT * sizeof(int);
   }
 };
 
@@ -118,11 +122,18 @@ template <int D> __global__ void __launch_bounds__(256) eq64_table_kernel(Sweep6
     const double C = 2.0 * M[kShA] * M[kQ0 + a] * c;
     if (a == 0) {
       E *= M[kDtTau] * M[kPre];
-      const double w = A.wv[j], w1 = w * c, w2 = w * c2;
+      // w c, w c^2 and w c^3, rounded once each (every velocity of the node carries
+      // that rounding, so it does not average out): c as c + cl (Knuth's TwoSum),
+      // products with their errors (FMA)
+      const double w = A.wv[j], U = M[kU0], cb = c - A.xi1[j], cl = (A.xi1[j] - (c - cb)) - (U + cb);
+      const double c2l = fma(2.0 * c, cl, fma(c, c, -c2));
+      const double h1 = w * c, w1 = h1 + fma(w, cl, fma(w, c, -h1));
+      const double h2 = w * c2, e2 = fma(w, c2l, fma(w, c2, -h2)), w2 = h2 + e2;
+      const double h3 = h2 * c, w3 = h3 + fma(h2, cl, fma(e2, c, fma(h2, c, -h3)));
       double2 *o = reinterpret_cast<double2 *>(A.tab0 + (ci * A.nvx[0] + j) * T0);
       o[0] = make_double2(E, C);
       o[1] = make_double2(z - ((D == 2) ? 2.0 : 2.5), w1);
-      o[2] = make_double2(w2, w2 * c);
+      o[2] = make_double2(w2, w3);
     } else {
       double2 *o = reinterpret_cast<double2 *>(A.tabp + (ci * (nt - A.nvx[0]) + j - A.nvx[0]) * TP);
       o[0] = make_double2(E, C);
@@ -200,6 +211,7 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double *hb = red + 2 * W64 * NM * 32 + warp * 2 * C::NH * KG; // inflow faces at this warp's tile's upwind edge,
   double *hd = hb + C::NH * KG;                                 // and the differences across them
+  int *low = reinterpret_cast<int *>(red + 2 * W64 * NM * 32 + W64 * 2 * C::NH * KG); // of acc: the sums' errors
   const int nx = A.n[0], ny = (D == 3) ? A.n[1] : 1, nl = A.n[LA];
   const int ntx = (nx + CX - 1) / CX, nty = (D == 3) ? (ny + 3) / 4 : 1;
   const int tile = blockIdx.x % (ntx * nty), rr = blockIdx.x / (ntx * nty);
@@ -212,7 +224,10 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
   const long long ps = (long long)nx * ny, col0 = ijk[0] + (long long)nx * ijk[1];
   const int npn = A.nvx[1] + ((D == 3) ? A.nvx[2] : 0); // nodes of the other axes
 
-  for (int e = threadIdx.x; e < M * NM * CT; e += 32 * W64) acc[e] = 0.0;
+  for (int e = threadIdx.x; e < M * NM * CT; e += 32 * W64) {
+    acc[e] = 0.0;
+    low[e] = 0;
+  }
   __syncthreads();
   int par = 0;
   const int b1 = min(A.nbatch, ((int)blockIdx.y + 1) * A.per);
@@ -342,7 +357,7 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
 
         // the cell's constants of this row
         const double *Mc = A.mac + c * kMac;
-        const double c0 = 1.0 - Mc[kDtTau], hT = (D == 2) ? Mc[kHalfT] : 0.0;
+        const double mt = -Mc[kDtTau], hT = (D == 2) ? Mc[kHalfT] : 0.0;
         const size_t ci = (size_t)(c - A.cbase);
         const double2 *t0 = reinterpret_cast<const double2 *>(A.tab0 + (ci * A.nvx[0] + g.kx) * T0);
         const double2 *tp = reinterpret_cast<const double2 *>(A.tabp + (ci * npn + ky) * TP);
@@ -377,8 +392,10 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
               // dt / tau times the equilibrium
               const double e = e0.x * Er, Cc = e0.y + Cr, t = e1.x + tr;
               const double H = fma(e, Cc * t, e);
-              n[0] = fma(c0, F[j][0], H);
-              if constexpr (D == 2) n[1] = fma(hT, fma(e, Cc, H), c0 * F[j][1]);
+              // the increments of relaxation and fluxes first; f joins them last, so
+              // that f^{n+1} is rounded once at its own size
+              n[0] = fma(mt, F[j][0], H);
+              if constexpr (D == 2) n[1] = fma(hT, fma(e, Cc, H), mt * F[j][1]);
 #pragma unroll
               for (int m = 0; m < NC; ++m) {
                 const double f = F[j][m];
@@ -428,7 +445,7 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
                 P[j][m] = zo;
                 Dd[j][m] = b;
                 F[j][m] = vz[m];
-                n[m] = fma(al, zin - zo, n[m]);
+                n[m] = fma(al, zin - zo, n[m]) + f;
               }
               if (fluid && own2) {
                 if constexpr (NC == 2)
@@ -489,13 +506,19 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
       }
       __syncthreads();
       // add the block's sums of this row (a buffer is written again two barriers later)
+      // and keep what the additions round away (Kahan's sum): one such sum takes all
+      // the groups of the block, a chain long enough to show in the heat flux.  The
+      // high word of the error is enough, and needs no conversion
       double *ar = acc + (p - ya) * NM * CT;
+      int *lr = low + (p - ya) * NM * CT;
       for (int e = threadIdx.x; e < NM * CT; e += 32 * W64) {
         const double *q = red + par * W64 * NM * 32 + (e / CT) * 32 + e % CT;
         static_assert(W64 == 4, "the pairwise sum below");
         auto at = [&](int w) { return (D == 2) ? q[w * NM * 32] + q[w * NM * 32 + 16] : q[w * NM * 32]; };
         const double v = (at(0) + at(1)) + (at(2) + at(3));
-        ar[e] += v;
+        const double y = v - __hiloint2double(lr[e], 0), s = ar[e], t = s + y;
+        lr[e] = __double2hiint((t - s) - y);
+        ar[e] = t;
       }
     }
   }
@@ -504,7 +527,7 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
     const int q = e % CT, m = (e / CT) % NM, p = ya + e / (CT * NM);
     const int x = x0 + q % CX, y = (D == 3) ? y0 + q / CX : 0;
     if (x < nx && y < ny)
-      A.part[((size_t)blockIdx.y * NM + m) * A.ncell + x + (long long)nx * y + ps * p] = acc[e];
+      A.part[((size_t)blockIdx.y * NM + m) * A.ncell + x + (long long)nx * y + ps * p] = acc[e] - __hiloint2double(low[e], 0);
   }
 }
 
@@ -595,48 +618,53 @@ void sweep64_groups(const Geom &G, std::vector<int> &out) {
   int negx = 0;
   while (negx < nx && xi(negx, 0, 0, 0) < 0.0) ++negx;
   for (int march = 0; march < 2; ++march) {
-    // x runs outermost: the four groups of a batch share their x nodes' tables
-    for (int part = 0; part < 2; ++part) {
-      const int lo = part ? negx : 0, hi = part ? nx : negx;
-      const int ng = (hi - lo + KG - 1) / KG;
-      for (int q = 0; q < ng; ++q) {
-        const int a = lo + (int)((long long)(hi - lo) * q / ng), b = lo + (int)((long long)(hi - lo) * (q + 1) / ng);
-        for (int kz = 0; kz < nz; ++kz)
-          for (int ky = 0; ky < ny; ++ky) {
-            const bool yneg = xi(0, ky, kz, 1) < 0.0, zneg = G.dim == 3 && xi(0, ky, kz, 2) < 0.0;
-            if ((G.dim == 3 ? zneg : yneg) != (march == 1)) continue;
-            Grp64 g{};
-            g.k[0] = a + nx * (ky + ny * kz);
-            g.k[1] = -1;
-            g.cnt = b - a;
-            g.kx = a;
-            g.ky[0] = g.ky[1] = ky;
-            g.kz = kz;
-            g.sgn = (part ? 0 : 1) | (yneg ? 2 : 0) | (zneg ? 4 : 0);
-            if (G.dim == 2 && ky + 1 < ny && (xi(0, ky + 1, kz, 1) < 0.0) == yneg) {
-              ++ky;
-              g.k[1] = a + nx * ky;
-              g.ky[1] = ky;
-            }
-            list[march].push_back(g);
-          }
+    // rows of the velocity grid marched this way (2D: pairs of one sign)
+    struct Row {
+      int ky[2], kz, sgn;
+    };
+    std::vector<Row> rows;
+    for (int kz = 0; kz < nz; ++kz)
+      for (int ky = 0; ky < ny; ++ky) {
+        const bool yneg = xi(0, ky, kz, 1) < 0.0, zneg = G.dim == 3 && xi(0, ky, kz, 2) < 0.0;
+        if ((G.dim == 3 ? zneg : yneg) != (march == 1)) continue;
+        Row r{{ky, -1}, kz, (yneg ? 2 : 0) | (zneg ? 4 : 0)};
+        if (G.dim == 2 && ky + 1 < ny && (xi(0, ky + 1, kz, 1) < 0.0) == yneg) r.ky[1] = ++ky;
+        rows.push_back(r);
       }
-    }
-    // the fill stands at the end of the first list and at the front of the second
+    if (march == 1) std::reverse(rows.begin(), rows.end()); // the opposite rows at the same places
+    // x runs outermost, a row's group of negative x and its mirror image next to
+    // each other: a batch adds them first, so that the sums of odd moments stay
+    // small (heat flux along x of a 16^2 box with 24^2 velocities: rms error 3.3e-17,
+    // 5.0e-17 with four groups of one sign to a batch)
+    const int lo[2] = {0, negx}, n[2] = {negx, nx - negx}, ng[2] = {(n[0] + KG - 1) / KG, (n[1] + KG - 1) / KG};
+    for (int i = 0; i < std::max(ng[0], ng[1]); ++i)
+      for (const Row &r : rows)
+        for (int part = 0; part < 2; ++part) {
+          if (i >= ng[part]) continue;
+          const int q = part ? ng[1] - 1 - i : i;
+          const int a = lo[part] + (int)((long long)n[part] * q / ng[part]);
+          const int b = lo[part] + (int)((long long)n[part] * (q + 1) / ng[part]);
+          Grp64 g{};
+          for (int h = 0; h < 2; ++h) {
+            const int ky = r.ky[h] < 0 ? r.ky[0] : r.ky[h];
+            g.ky[h] = ky;
+            g.k[h] = (r.ky[h] < 0) ? -1 : a + nx * (ky + ny * r.kz);
+          }
+          g.cnt = b - a;
+          g.kx = a;
+          g.kz = r.kz;
+          g.sgn = (part ? 0 : 1) | r.sgn;
+          list[march].push_back(g);
+        }
     const Grp64 none{{0, -1}, 0, 0, {0, 0}, 0, march ? (G.dim == 3 ? 4 : 2) : 0};
-    const size_t fill = (W64 - list[march].size() % W64) % W64;
-    list[march].insert(march ? list[march].begin() : list[march].end(), fill, none);
+    list[march].insert(list[march].end(), (W64 - list[march].size() % W64) % W64, none);
   }
-  // the batches of the first list in turn with those of the second backwards,
-  // which hold the opposite velocities: the sums of odd moments stay small as
-  // they grow, and so do their roundings (heat flux of the 128^2 lid-driven
-  // cavity against 64-bit tensors: 1.0e-13 relative with one list after the
-  // other, 6.9e-14 in turn)
+  // the batches of the two lists, which hold opposite velocities, in turn: the sums
+  // of odd moments stay small as they grow, and so do their roundings
   const size_t nb[2] = {list[0].size() / W64, list[1].size() / W64};
-  for (size_t b = 0; b < std::max(nb[0], nb[1]); ++b) {
-    if (b < nb[0]) gs.insert(gs.end(), list[0].begin() + b * W64, list[0].begin() + (b + 1) * W64);
-    if (b < nb[1]) gs.insert(gs.end(), list[1].end() - (b + 1) * W64, list[1].end() - b * W64);
-  }
+  for (size_t b = 0; b < std::max(nb[0], nb[1]); ++b)
+    for (int march = 0; march < 2; ++march)
+      if (b < nb[march]) gs.insert(gs.end(), list[march].begin() + b * W64, list[march].begin() + (b + 1) * W64);
   out.resize(gs.size() * sizeof(Grp64) / sizeof(int));
   std::copy(reinterpret_cast<const int *>(gs.data()), reinterpret_cast<const int *>(gs.data()) + out.size(), out.begin());
 }
