@@ -157,8 +157,9 @@ typedef struct {
   int precision;
   long long steps_done;
   size_t device_bytes;
-  int sweep_variant; /* 0: FP64 sweep (sweep64.cu; FP32 without TMA: kernels.cu), 1: TMA-staged 2D
-                        FP32 sweep (sweep_tma.cu), 2: TMA-staged 3D FP32 sweep (sweep3d_tma.cu),
+  int sweep_variant; /* 0: FP64 sweep (sweep64.cu; the smallest FP64 grids, and FP32 without TMA:
+                        kernels.cu), 1: TMA-staged 2D FP32 sweep (sweep_tma.cu), 2: TMA-staged 3D
+                        FP32 sweep (sweep3d_tma.cu),
                         3: the sweep of a tree-refined grid (FP32 tree_sweep.cu, FP64 kernels.cu) */
 } ibdvm_info;
 

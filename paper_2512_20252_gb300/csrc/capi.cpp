@@ -742,7 +742,7 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
     int nchunk = static_cast<int>(std::min<long long>(kblocks, std::max<long long>(1, (4 * 152 + cell_blocks - 1) / cell_blocks)));
     ctx->kloop = (kblocks + nchunk - 1) / nchunk;
     ctx->nchunk = (kblocks + ctx->kloop - 1) / ctx->kloop;
-    const bool fp64_sweep = ctx->precision == IBDVM_FP64 && !tree;
+    const bool fp64_sweep = ctx->precision == IBDVM_FP64 && !tree && !sweep64_direct(G);
     if (fp64_sweep) ctx->nchunk = sweep64_nchunk(G);
     const int NW = G.dim + 2;
     const int NM = nmoments(G.dim);

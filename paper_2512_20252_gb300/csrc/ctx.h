@@ -98,7 +98,7 @@ struct ibdvm_ctx {
   uint8_t *ctype = nullptr;
   uint8_t *cmask = nullptr;  // per cell: ghost neighbour per face (bit 2a + (s > 0)), 64 = not fluid
   int *dslot = nullptr, *dlinks = nullptr;
-  ibdvm::Sweep64Plan plan64; // FP64 on a uniform grid (sweep64.cu)
+  ibdvm::Sweep64Plan plan64; // FP64 on a uniform grid (sweep64.cu; no batches: the sweep of kernels.cu)
   // TMA sweep of 2D FP32 cases (sweep_tma.cu)
   bool use_tma = false;
   float *partf = nullptr;    // FP32 moment partial sums [nchunk][9][ncell]
@@ -211,6 +211,8 @@ cudaError_t tma_sweep_launch(ibdvm_ctx *ctx);
 // FP64 sweep of uniform grids (sweep64.cu): the chunks of its moment sums, the
 // bytes of its tables (fewer when memory is short), its set-up (groups and
 // axis nodes for the caller to upload) and one step's launches
+// (sweep64_direct: the sweep of kernels.cu takes the case instead)
+bool sweep64_direct(const Geom &G);
 int sweep64_nchunk(const Geom &G);
 size_t sweep64_table_bytes(const Geom &G);
 cudaError_t sweep64_prepare(ibdvm_ctx *ctx, std::vector<int> &grp, std::vector<double> &nodes);

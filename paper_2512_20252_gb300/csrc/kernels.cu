@@ -17,7 +17,8 @@
 //                       (cell, velocity), van Leer limited upwind face values (Eqs.
 //                       reconstruction, limiter), flux divergence, Shakhov relaxation
 //                       with the reduced equilibria, forward Euler, and the velocity
-//                       moments of the new state reduced per cell (FP64: sweep64.cu).
+//                       moments of the new state reduced per cell; in FP64 the
+//                       smallest grids (the others: sweep64.cu).
 //   finalize_kernel     moments -> W, T, q, tau per cell; the residual (Sec. 4, FP64).
 //   forces_kernel       momentum and energy through the donor-ghost faces (FP64).
 //
@@ -2386,8 +2387,9 @@ cudaError_t launch_sweep(ibdvm_ctx *ctx) {
     {
       Timed tm(ctx, kKSweep);
       if constexpr (std::is_same<T, double>::value) {
-        ctx->kernel_launches[kKSweep] += ctx->tree ? 1 : sweep64_launches(ctx);
-        e = ctx->tree ? tree_sweep_t<T, D>(ctx) : sweep64_launch(ctx);
+        const bool faces = !ctx->tree && ctx->plan64.nbatch > 0;
+        ctx->kernel_launches[kKSweep] += faces ? sweep64_launches(ctx) : 1;
+        e = ctx->tree ? tree_sweep_t<T, D>(ctx) : faces ? sweep64_launch(ctx) : sweep_t<T, D>(ctx, 1, 1);
       } else {
         // (a tree: the regular leaves and the others)
         ctx->kernel_launches[kKSweep] += ctx->tree ? (ctx->tree_nreg > 0) + (ctx->tree_nreg < ctx->ncell) : 1;

@@ -608,6 +608,17 @@ int slab_rows(const Geom &G) {
 
 } // namespace
 
+// Where the direct sweep (sweep_kernel: a thread per cell and velocity, every face
+// twice) is the faster one.  Its blocks are four cells and 64 velocities: up to one
+// per SM it takes 25 us whatever they hold, less than a row and a march's start here
+// (sweep and moments of 4^2 cells x 24^2 velocities 58 us direct, 66 here, 12^2 x 16^2
+// 59 / 67; in two rounds 6^3 x 6^3 93 / 77).  And 2D grids of four columns leave three
+// lanes of four idle here (4 x 512 x 24^2: 522 / 603; of five columns 696 / 607).
+bool sweep64_direct(const Geom &G) {
+  const long long blocks = ((G.ncell + 3) / 4) * ((G.nv + 63) / 64);
+  return blocks <= 152 || (G.dim == 2 && G.n[0] <= 4);
+}
+
 void sweep64_groups(const Geom &G, std::vector<int> &out) {
   // groups of at most KG nodes of one sign along x, as even as they go; in 2D
   // two y rows of one sign each; the groups of one march sign in one list, filled
@@ -673,15 +684,15 @@ void sweep64_groups(const Geom &G, std::vector<int> &out) {
 // two blocks each.  A block's work is its rows and the march's start (about half
 // a row) times its batches; two blocks of an SM keep its FP64 pipe 86% busy, one
 // alone 65% (measured), so a last round of at most one block per SM counts its
-// work once over 0.65 and any other round twice over 0.86.
+// work once over 0.65 and any other round twice over 0.86.  A chunk costs the
+// finalize kernel of a small grid 0.75 to 0.9 us, 0.08 rows of a batch.
 void sweep64_tiling(const Geom &G, int nbatch, int &rows, int &per) {
   const int D = G.dim, nl = slab_rows(G);
   const long long tiles = (D == 2) ? (G.n[0] + 15) / 16 : (long long)((G.n[0] + 7) / 8) * ((G.n[1] + 3) / 4);
   const int maxr = (D == 2) ? Cfg64<2>::MAXROWS : Cfg64<3>::MAXROWS;
   double best = 1e300;
-  for (int nr = (nl + maxr - 1) / maxr; nr <= nl; ++nr) {
-    const int r = (nl + nr - 1) / nr;
-    if (r < 4 && nr > (nl + maxr - 1) / maxr) break;
+  for (int most = std::min(maxr, nl); most >= 1; --most) {
+    const int r = (nl + (nl + most - 1) / most - 1) / ((nl + most - 1) / most);
     const long long tr = tiles * ((nl + r - 1) / r);
     for (int pb = nbatch; pb >= 1; --pb) {
       const int nch = (nbatch + pb - 1) / pb;
@@ -689,7 +700,7 @@ void sweep64_tiling(const Geom &G, int nbatch, int &rows, int &per) {
       const long long blocks = tr * nch;
       const long long full = blocks / 304, rem = blocks % 304;
       const double rounds = full * (2.0 / 0.86) + (rem == 0 ? 0.0 : rem <= 152 ? 1.0 / 0.65 : 2.0 / 0.86);
-      const double cost = rounds * pb * (r + 0.5) + 0.02 * nch;
+      const double cost = rounds * pb * (r + 0.5) + 0.08 * nch;
       if (cost < best * (1.0 - 1e-9)) {
         best = cost;
         rows = r;
