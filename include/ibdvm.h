@@ -172,6 +172,9 @@ typedef struct {
    no body.  cuda_stream is a cudaStream_t (NULL = the legacy default stream);
    the context keeps it for every launch.  The context owns all device memory
    it allocates (ibdvm_destroy frees it); descriptors are copied, not kept.
+   FP64 cases also hold tables of their sweep: a share of what memory the case
+   leaves free (1/64, 256 MB at most), which later calls on the context
+   (ibdvm_set_body, ibdvm_set_domain, ...) take back where they need it.
    Errors: IBDVM_E_INVAL (bad descriptor), IBDVM_E_NOMEM (device memory short:
    checked against cudaMemGetInfo before allocating), IBDVM_E_CUDA. */
 ibdvm_status ibdvm_create_grid(const ibdvm_grid_desc *grid, const ibdvm_vgrid_desc *vgrid,

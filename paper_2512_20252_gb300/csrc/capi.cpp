@@ -38,11 +38,38 @@ template <typename T> void cfree_t(T *&p) {
   p = nullptr;
 }
 
+void drop_graphs(ibdvm_ctx *ctx);
+
+// The tables of the FP64 sweep yield to what else the case needs: halves them where
+// that can make room for `bytes`
+bool give_back(ibdvm_ctx *ctx, size_t bytes) {
+  const Sweep64Plan &pl = ctx->plan64;
+  size_t freeb = 0, totb = 0;
+  if (!pl.tab || pl.slab <= 1 || cudaMemGetInfo(&freeb, &totb) != cudaSuccess ||
+      freeb + pl.tab_bytes < bytes + pl.tab_bytes / pl.slab || cudaStreamSynchronize(ctx->stream) != cudaSuccess)
+    return false;
+  drop_graphs(ctx); // they hold the tables' address and slabs
+  ctx->dev_bytes -= pl.tab_bytes;
+  const cudaError_t e = sweep64_tables(ctx, pl.slab / 2);
+  ctx->dev_bytes += pl.tab_bytes;
+  return e == cudaSuccess;
+}
+
+cudaError_t grab(ibdvm_ctx *ctx, void **p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  while (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    if (!give_back(ctx, bytes)) break;
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
 // cudaMalloc with bookkeeping; throws Fail on error
 template <typename T> T *dalloc(ibdvm_ctx *ctx, size_t count, const char *what) {
   void *p = nullptr;
   size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
-  cudaError_t e = cudaMalloc(&p, bytes);
+  cudaError_t e = grab(ctx, &p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     ctx->err = std::string("device allocation of ") + what + " (" + std::to_string(bytes) +
@@ -751,12 +778,13 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
     const size_t need = 2 * fbytes + static_cast<size_t>(ctx->ncell) * (ctx->nvp / 64 + 1) * 4 * (G.dim == 2 ? 9 : 14) +
                         static_cast<size_t>(ctx->ncell) *
                                          (kMac * ctx->esize + 2 * (NW + G.dim) * 8 + ctx->nchunk * NM * 8 + 8);
+    const size_t row = fp64_sweep ? sweep64_row_bytes(G) : 0; // the least of its tables
     int dev = 0;
     check(ctx, cudaGetDevice(&dev), "cudaGetDevice");
     size_t freeb = 0, totb = 0;
     check(ctx, cudaMemGetInfo(&freeb, &totb), "cudaMemGetInfo");
-    if (need > freeb) {
-      ctx->err = "the case needs " + std::to_string(need) + " bytes of device memory, " +
+    if (need + row > freeb) {
+      ctx->err = "the case needs " + std::to_string(need + row) + " bytes of device memory, " +
                  std::to_string(freeb) + " are free";
       throw Fail{IBDVM_E_NOMEM};
     }
@@ -800,22 +828,6 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
       ctx->oct_sign = dalloc<uint8_t>(ctx, sign.size(), "chunk signs");
       upload(ctx, ctx->oct_const, vconst, "upload velocity constants");
       upload(ctx, ctx->oct_sign, sign, "upload chunk signs");
-    }
-    if (fp64_sweep) {
-      std::vector<int> grp;
-      std::vector<double> nodes;
-      cudaError_t e = sweep64_prepare(ctx, grp, nodes);
-      if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        ctx->err = "device allocation of the equilibrium tables failed";
-        throw Fail{IBDVM_E_NOMEM};
-      }
-      check(ctx, e, "FP64 sweep set-up");
-      ctx->dev_bytes += ctx->plan64.tab_bytes;
-      ctx->plan64.grp = dalloc<int>(ctx, grp.size(), "velocity groups");
-      ctx->plan64.nodes = dalloc<double>(ctx, nodes.size(), "velocity nodes");
-      upload(ctx, ctx->plan64.grp, grp, "upload velocity groups");
-      upload(ctx, ctx->plan64.nodes, nodes, "upload velocity nodes");
     }
     // the TMA sweeps of FP32 cases
     if (!tma_off && (tma_sweep_applicable(ctx) || tma3_sweep_applicable(ctx))) {
@@ -886,6 +898,23 @@ static ibdvm_status create_ctx(const ibdvm_grid_desc *grid, const ibdvm_tree_des
     for (int i = 0; i < 2; ++i)
       check(ctx, cudaMemsetAsync(ctx->W[i], 0, static_cast<size_t>(NW + G.dim) * ctx->ncell * 8, ctx->stream), "clear");
     upload_body(ctx);
+    // the tables of the FP64 sweep come last: they take less where less is left
+    if (fp64_sweep) {
+      std::vector<int> grp;
+      std::vector<double> nodes;
+      cudaError_t e = sweep64_prepare(ctx, grp, nodes);
+      if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        ctx->err = "device allocation of the equilibrium tables failed";
+        throw Fail{IBDVM_E_NOMEM};
+      }
+      check(ctx, e, "FP64 sweep set-up");
+      ctx->dev_bytes += ctx->plan64.tab_bytes;
+      ctx->plan64.grp = dalloc<int>(ctx, grp.size(), "velocity groups");
+      ctx->plan64.nodes = dalloc<double>(ctx, nodes.size(), "velocity nodes");
+      upload(ctx, ctx->plan64.grp, grp, "upload velocity groups");
+      upload(ctx, ctx->plan64.nodes, nodes, "upload velocity nodes");
+    }
     check(ctx, launch_init_state(ctx), "init kernel");
     refresh_moments(ctx);
     st = status_of_flags(ctx, read_flags(ctx));
@@ -1009,7 +1038,7 @@ ibdvm_status ibdvm_set_domain(ibdvm_ctx *ctx, const ibdvm_domain_desc *d) {
       }
     }
     const void *src = t2.empty() ? static_cast<const void *>(t.data()) : t2.data();
-    const bool ok = cudaMalloc(&halo, halo_bytes) == cudaSuccess && cudaMalloc(&tab, tab_bytes) == cudaSuccess;
+    const bool ok = grab(ctx, &halo, halo_bytes) == cudaSuccess && grab(ctx, &tab, tab_bytes) == cudaSuccess;
     cudaError_t e = ok ? cudaMemcpyAsync(tab, src, tab_bytes, cudaMemcpyHostToDevice, ctx->stream) : cudaSuccess;
     if (ok && e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream); // the host table goes out of scope
     if (!ok || e != cudaSuccess) {

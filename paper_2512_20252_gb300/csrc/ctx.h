@@ -53,6 +53,7 @@ constexpr unsigned kNotFluidCell = 64;
 struct Sweep64Plan {
   int nbatch = 0, per = 0; // batches of velocity groups, per chunk of the moment sums
   int rows = 0, slab = 0;  // rows of the last axis per block, and per launch
+  int most = 0;            // rows per block where a launch has as many
   int nnode = 0;           // velocity nodes of all axes
   int *grp = nullptr;      // the groups
   double *nodes = nullptr; // [3][nnode]: component, dt |xi| / dx, width
@@ -209,12 +210,14 @@ int tma_sweep_nchunk(const ibdvm_ctx *ctx);
 cudaError_t tma_sweep_prepare(ibdvm_ctx *ctx);
 cudaError_t tma_sweep_launch(ibdvm_ctx *ctx);
 // FP64 sweep of uniform grids (sweep64.cu): the chunks of its moment sums, the
-// bytes of its tables (fewer when memory is short), its set-up (groups and
-// axis nodes for the caller to upload) and one step's launches
+// bytes of its tables (fewer when memory is short) and of a row of them, its set-up
+// (groups and axis nodes for the caller to upload), its tables and one step's launches
 // (sweep64_direct: the sweep of kernels.cu takes the case instead)
 bool sweep64_direct(const Geom &G);
 int sweep64_nchunk(const Geom &G);
 size_t sweep64_table_bytes(const Geom &G);
+size_t sweep64_row_bytes(const Geom &G);
+cudaError_t sweep64_tables(ibdvm_ctx *ctx, int slab);
 cudaError_t sweep64_prepare(ibdvm_ctx *ctx, std::vector<int> &grp, std::vector<double> &nodes);
 int sweep64_launches(const ibdvm_ctx *ctx);
 cudaError_t sweep64_launch(ibdvm_ctx *ctx);

@@ -601,6 +601,8 @@ size_t row_bytes(const Geom &G) {
 // Tables of at most this size: a larger grid is swept slab by slab (rows of the
 // last axis), with one table for all
 constexpr size_t kTableBytes = size_t(256) << 20;
+// and of at most this share of the memory that the rest of the case leaves free
+constexpr size_t kTableShare = 64;
 
 int slab_rows(const Geom &G) {
   return (int)std::min<size_t>(G.n[G.dim - 1], std::max<size_t>(1, kTableBytes / row_bytes(G)));
@@ -720,8 +722,31 @@ int sweep64_nchunk(const Geom &G) {
   return (nbatch + per - 1) / per;
 }
 
-size_t sweep64_table_bytes(const Geom &G) {
-  return row_bytes(G) * slab_rows(G);
+size_t sweep64_table_bytes(const Geom &G) { return row_bytes(G) * slab_rows(G); }
+size_t sweep64_row_bytes(const Geom &G) { return row_bytes(G); }
+
+// The tables of `slab` rows (one at least), fewer where memory is short, in place
+// of those there are; no work of the stream may use them
+cudaError_t sweep64_tables(ibdvm_ctx *ctx, int slab) {
+  const Geom &G = ctx->geom;
+  Sweep64Plan &pl = ctx->plan64;
+  if (pl.tab) cudaFree(pl.tab);
+  pl.tab = nullptr;
+  pl.tab_bytes = 0;
+  const size_t rb = row_bytes(G);
+  cudaError_t e;
+  for (slab = std::max(slab, 1);; slab = (slab + 1) / 2) {
+    void *p = nullptr;
+    e = cudaMalloc(&p, rb * slab);
+    pl.tab = static_cast<double *>(p);
+    if (e == cudaSuccess || slab == 1) break;
+    cudaGetLastError();
+  }
+  pl.slab = slab;
+  if (e != cudaSuccess) return e;
+  pl.tab_bytes = rb * slab;
+  pl.rows = std::min(pl.most, slab);
+  return cudaSuccess;
 }
 
 cudaError_t sweep64_prepare(ibdvm_ctx *ctx, std::vector<int> &grp, std::vector<double> &nodes) {
@@ -729,7 +754,7 @@ cudaError_t sweep64_prepare(ibdvm_ctx *ctx, std::vector<int> &grp, std::vector<d
   Sweep64Plan &pl = ctx->plan64;
   sweep64_groups(G, grp);
   pl.nbatch = (int)(grp.size() * sizeof(int) / sizeof(Grp64)) / W64;
-  sweep64_tiling(G, pl.nbatch, pl.rows, pl.per);
+  sweep64_tiling(G, pl.nbatch, pl.most, pl.per);
   // axis nodes: the component, dt |xi| / dx and the node's width
   pl.nnode = G.nvx[0] + G.nvx[1] + ((G.dim == 3) ? G.nvx[2] : 0);
   nodes.assign(3 * (size_t)pl.nnode, 0.0);
@@ -742,21 +767,10 @@ cudaError_t sweep64_prepare(ibdvm_ctx *ctx, std::vector<int> &grp, std::vector<d
       nodes[2 * (size_t)pl.nnode + o] = G.bhi[3 * (i * st) + a] - G.blo[3 * (i * st) + a];
     }
   }
-  // the table: as many rows as fit its size, fewer when memory is short
-  const size_t rb = row_bytes(G);
-  int slab = slab_rows(G);
-  cudaError_t e;
-  for (;; slab = (slab + 1) / 2) {
-    void *p = nullptr;
-    e = cudaMalloc(&p, rb * slab);
-    pl.tab = static_cast<double *>(p);
-    if (e == cudaSuccess || slab == 1) break;
-    cudaGetLastError();
-  }
+  size_t freeb = 0, totb = 0;
+  cudaError_t e = cudaMemGetInfo(&freeb, &totb);
+  if (e == cudaSuccess) e = sweep64_tables(ctx, (int)std::min<size_t>(slab_rows(G), freeb / kTableShare / row_bytes(G)));
   if (e != cudaSuccess) return e;
-  pl.slab = slab;
-  pl.tab_bytes = rb * slab;
-  pl.rows = std::min(pl.rows, slab);
   e = (G.dim == 2) ? cudaFuncSetAttribute(sweep64_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)Cfg64<2>::smem(Cfg64<2>::MAXROWS))
                    : cudaFuncSetAttribute(sweep64_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -769,6 +783,9 @@ int sweep64_launches(const ibdvm_ctx *ctx) {
   return 2 * ((nl + ctx->plan64.slab - 1) / ctx->plan64.slab);
 }
 
-cudaError_t sweep64_launch(ibdvm_ctx *ctx) { return (ctx->dim == 2) ? launch64<2>(ctx) : launch64<3>(ctx); }
+cudaError_t sweep64_launch(ibdvm_ctx *ctx) {
+  if (!ctx->plan64.tab) return cudaErrorMemoryAllocation;
+  return (ctx->dim == 2) ? launch64<2>(ctx) : launch64<3>(ctx);
+}
 
 } // namespace ibdvm
