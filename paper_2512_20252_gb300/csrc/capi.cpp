@@ -1477,7 +1477,39 @@ const char *ibdvm_geom_last_error(void) { return g_geom_err.c_str(); }
 } // extern "C"
 
 namespace ibdvm {
-size_t estimate_ctx_bytes(const ibdvm_grid_desc *grid, const ibdvm_vgrid_desc *vgrid, const ibdvm_gas_desc *gas) {
+namespace {
+// An upper bound of a body's links.  Every link crosses the body's surface on a grid
+// line; a line crosses a convex body twice at most (a half-space once), a polygon
+// once per edge that spans it.
+double link_bound(const Geom &G, const ibdvm_body_desc &b) {
+  if (b.kind == IBDVM_BODY_NONE) return 0.0;
+  double all = 0.0, nl = 0.0; // lines of the grid; links
+  for (int a = 0; a < G.dim; ++a) {
+    double lines = 1.0, box = 1.0;
+    for (int c = 0; c < G.dim; ++c) {
+      if (c == a) continue;
+      const double half = (b.kind == IBDVM_BODY_ELLIPSE) ? std::max(b.radii[0], b.radii[1]) : b.radii[0];
+      lines *= G.n[c];
+      box *= std::max(0.0, std::min<double>(G.n[c], 2.0 * half / G.dx[c] + 2.0));
+    }
+    all += lines;
+    nl += 2.0 * box;
+  }
+  if (b.kind == IBDVM_BODY_HALFSPACE) return all;
+  if (b.kind != IBDVM_BODY_POLYGON) return nl;
+  nl = 0.0;
+  for (int e = 0; b.verts && e < b.nverts; ++e)
+    for (int c = 0; c < 2; ++c) { // lines of cell centres from one end to the other
+      const double u = (b.verts[2 * e + c] - G.lo[c]) / G.dx[c] - 0.5;
+      const double v = (b.verts[2 * ((e + 1) % b.nverts) + c] - G.lo[c]) / G.dx[c] - 0.5;
+      nl += std::max(0.0, std::floor(std::max(u, v) + 1e-9) - std::ceil(std::min(u, v) - 1e-9) + 1.0);
+    }
+  return std::isfinite(nl) ? nl : all; // (a polygon that will be refused)
+}
+} // namespace
+
+size_t estimate_ctx_bytes(const ibdvm_grid_desc *grid, const ibdvm_vgrid_desc *vgrid, const ibdvm_gas_desc *gas,
+                          const ibdvm_body_desc *body) {
   Geom G;
   std::string err;
   if (!build_grid(*grid, *vgrid, *gas, G, err)) return 0;
@@ -1493,14 +1525,14 @@ size_t estimate_ctx_bytes(const ibdvm_grid_desc *grid, const ibdvm_vgrid_desc *v
   size_t b = 2 * nc * nvp * G.ncomp * es;                               // f^n, f^{n+1}
   b += nc * (nvp / 64 + 1) * 4 * NM;                                     // FP32 moment partial sums
   size_t chunks = nvp / 64 + 1;
-  if (gas->precision == IBDVM_FP64) { // the FP64 sweep's chunks and tables
+  if (gas->precision == IBDVM_FP64 && !sweep64_direct(G)) { // the FP64 sweep's chunks and tables
     chunks = std::max(chunks, static_cast<size_t>(sweep64_nchunk(G)));
     b += sweep64_table_bytes(G);
   }
   b += nc * (kMac * es + 2 * (NW + D) * 8 + chunks * NM * 8 + 16); // per-cell state, FP64 sums
-  // the ghost band: at most D n^(D-1) links for a body that fits the domain
-  const double nl = D * std::pow(static_cast<double>(nc), (D - 1.0) / D);
-  b += static_cast<size_t>(nl) * (nvp * ((3 + 3 * D / 2.0) * G.ncomp * es + 16 + es) + 512);
+  // the ghost band, with half as many surface cells again as links
+  const double nl = body ? link_bound(G, *body) : 0.0;
+  b += static_cast<size_t>(nl * (nvp * ((3 + 3 * D / 2.0) * G.ncomp * es + 16 + es) + 512));
   return b + nvp * 64 + (1u << 20);
 }
 

@@ -316,8 +316,9 @@ void batch_detach(ibdvm_ctx *ctx);
 // waits for them and reads every member's residual and status
 ibdvm_status batch_enqueue(ibdvm_batch *b, int nsteps);
 ibdvm_status batch_collect(ibdvm_batch *b, double *residuals, int *statuses);
-// capi.cpp: an upper estimate of the device bytes of a context (before its body is placed)
-size_t estimate_ctx_bytes(const ibdvm_grid_desc *grid, const ibdvm_vgrid_desc *vgrid, const ibdvm_gas_desc *gas);
+// capi.cpp: an upper estimate of the device bytes of a context with a body (null: none); 0: invalid
+size_t estimate_ctx_bytes(const ibdvm_grid_desc *grid, const ibdvm_vgrid_desc *vgrid, const ibdvm_gas_desc *gas,
+                          const ibdvm_body_desc *body);
 // capi.cpp: F[3], Q, CD, CL (each nullable) from the force sums h[4] of ctx
 void force_outputs(const ibdvm_ctx *ctx, const double *h, double *F, double *Q, double *CD, double *CL);
 

@@ -97,7 +97,7 @@ int admit(ibdvm_server *s) {
     if (s->d.sequential_fp64 && !s->active.empty()) break;
     if (s->d.max_active > 0 && static_cast<int>(s->active.size()) >= s->d.max_active) break;
     Req *q = s->queue.front();
-    const size_t est = estimate_ctx_bytes(&q->grid, &q->vgrid, &q->gas);
+    const size_t est = estimate_ctx_bytes(&q->grid, &q->vgrid, &q->gas, q->has_body ? &q->body : nullptr);
     if (!s->active.empty() && s->used + est > s->budget) break; // wait for memory to free up
     s->queue.pop_front();
     const int di = q->grid.dim == 3 ? 1 : 0;
@@ -117,7 +117,6 @@ int admit(ibdvm_server *s) {
     }
     q->ctx = ctx;
     if (q->has_body) {
-      q->body.verts = q->verts.empty() ? nullptr : q->verts.data();
       st = ibdvm_set_body(ctx, &q->body);
       if (st != IBDVM_OK) {
         finish(s, q, st);
@@ -186,7 +185,7 @@ ibdvm_status ibdvm_server_submit(ibdvm_server *s, const ibdvm_grid_desc *grid, c
         q->vgrid.nodes[a] = q->vnodes[a].empty() ? nullptr : q->vnodes[a].data();
       }
     q->gas.precision = s->d.sequential_fp64 ? IBDVM_FP64 : IBDVM_MIXED;
-    if (estimate_ctx_bytes(&q->grid, &q->vgrid, &q->gas) == 0) {
+    if (estimate_ctx_bytes(&q->grid, &q->vgrid, &q->gas, nullptr) == 0) {
       delete q;
       s->err = "invalid grid, velocity grid or gas descriptor";
       return IBDVM_E_INVAL;
@@ -195,6 +194,7 @@ ibdvm_status ibdvm_server_submit(ibdvm_server *s, const ibdvm_grid_desc *grid, c
       q->body = *body;
       q->has_body = true;
       if (body->verts && body->nverts > 0) q->verts.assign(body->verts, body->verts + 2 * body->nverts);
+      q->body.verts = q->verts.empty() ? nullptr : q->verts.data(); // the request's own copy
     }
     q->id = s->next_id++;
     q->r.id = q->id;
