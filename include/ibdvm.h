@@ -473,8 +473,9 @@ ibdvm_status ibdvm_batch_forces(ibdvm_batch *b, double *F, double *Q, double *CD
 
 /* Tiling of the sweep's work items.  rows: target rows (3D: planes) per item
    (0 = whole columns).  Until a tiling is set or tuned rows reads 0 and the
-   items are whole columns in 3D and about 64 rows in 2D.  kpt (0, 2 or 4) is accepted and has no effect: every
-   member's sweep takes the velocity chunks of its orthant layout (2D: 192,
+   items are whole columns in 3D, and in 2D whole columns where these are many and
+   about 64 rows where they are few.  kpt (0, 2 or 4) is accepted and has no
+   effect: every member's sweep takes the velocity chunks of its orthant layout (2D: 192,
    128 or 64 velocities; 3D: 256 or 128), and get_tiling reports the
    velocities per lane of the first member's chunk (chunk / 32; 0 without
    members), the number of work items, the persistent grid and whether graphs
@@ -485,8 +486,8 @@ typedef struct {
 ibdvm_status ibdvm_batch_set_tiling(ibdvm_batch *b, int rows, int kpt);
 ibdvm_status ibdvm_batch_get_tiling(const ibdvm_batch *b, ibdvm_batch_tiling *out);
 
-/* Autotuner: for each candidate tiling (rows in {16, 32, 64, 128, whole
-   columns}) times steps_per_trial batched steps (even, >= 2) with CUDA
+/* Autotuner: for each candidate tiling (rows in {16, 32, 128, whole columns},
+   and the items of a batch without a tiling) times steps_per_trial batched steps (even, >= 2) with CUDA
    events on the batch's stream, after one untimed pair of steps, and keeps
    the fastest.  The trials are real steps: every member advances
    5 x (steps_per_trial + 2) steps.  best_ms (nullable) receives

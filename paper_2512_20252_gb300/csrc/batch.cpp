@@ -477,18 +477,23 @@ ibdvm_status ibdvm_batch_tune(ibdvm_batch *b, int steps_per_trial, double *best_
     b->err = "the batch has no members";
     return IBDVM_E_STATE;
   }
-  const int rows_c[5] = {16, 32, 64, 128, 0};
+  const int rows_c[5] = {-1, 16, 32, 128, 0}; // (-1: the items of a batch without a tiling)
   cudaEvent_t e0, e1;
   bcheck(b, cudaEventCreate(&e0), "create event");
   bcheck(b, cudaEventCreate(&e1), "create event");
   double best = 1e300;
-  int best_rows = b->rows;
+  const int rows0 = b->rows;
+  const bool tiled0 = b->tiled;
+  int best_rows = -1;
+  auto tiling = [&](int rows, bool tiled) {
+    b->rows = rows;
+    b->tiled = tiled;
+    b->dirty = true;
+  };
   ibdvm_status st = IBDVM_OK;
   try {
     for (int r : rows_c) {
-      b->rows = r;
-      b->tiled = true;
-      b->dirty = true;
+      tiling(std::max(r, 0), r >= 0);
       build(b);
       bcheck(b, cudaMemsetAsync(b->d_flags, 0, b->members.size() * sizeof(int), b->stream), "clear flags");
       advance(b, 2); // warm-up pair: captures the graphs of this tiling
@@ -508,12 +513,12 @@ ibdvm_status ibdvm_batch_tune(ibdvm_batch *b, int steps_per_trial, double *best_
   } catch (const BFail &) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    tiling(rows0, tiled0);
     throw;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  b->rows = best_rows;
-  b->dirty = true;
+  tiling(std::max(best_rows, 0), best_rows >= 0);
   build(b);
   if (best_ms) *best_ms = best;
   return IBDVM_OK;

@@ -744,12 +744,17 @@ void tma_batch_free(SweepTables &t) {
 // us, 4 of 140^2..324^2 1800 / 1114 / 1116 / 1173 / 1234 / 1470, 8 of 79^2..334^2
 // 3491 / 3420 / 3317 / 3308 / 3336 / 3380, 12 of 108^2..330^2 3888 / 3717 / 3614 /
 // 3565 / 3625 / 3716, 16 of 83^2..381^2 4600 / 4730 / 4565 / 4596 / 4569 / 4619.
+// A width with kWholeItems columns or more per resident block keeps them whole (step
+// of 24 members 7477 us, 7505 in 64 rows; 32: 10533 and 10772; 48: 14921 and 15400;
+// with a limit of 10 the first two take 7557 and 10683, with 4 twelve members 4441
+// for 4404).
 // 3D keeps whole columns, whose items are many: 2 members of 33^3 and 40^3 cells
 // 2391 us whole, 2465 in 24 or 32 planes; 4 of 42^3..58^3 13368 and 13887 (32).
 constexpr int kAutoRows = 64;
+constexpr int kWholeItems = 6;
 
 // rows > 0: target rows (3D: planes) of an item; 0: whole columns; < 0: no tiling
-// was set (2D: about kAutoRows rows; 3D: whole columns)
+// was set (2D: about kAutoRows rows where columns are few; 3D: whole columns)
 cudaError_t tma_batch_build(const std::vector<ibdvm_ctx *> &cases, const std::vector<int> &kpt, int rows,
                             int *flags, SweepTables &t, cudaStream_t s) {
   (void)kpt; // the chunk of every member is that of its velocity layout
@@ -761,10 +766,31 @@ cudaError_t tma_batch_build(const std::vector<ibdvm_ctx *> &cases, const std::ve
   std::vector<Oct2Args> args(2 * n);
   std::vector<CUtensorMap> maps(2 * n);
   std::vector<WorkItem> items;
+  // the launches, one per chunk width (velocities per lane 6, 4, 2): resident blocks
+  // and columns
+  static const int kVpl[3] = {6, 4, 2};
+  int dev = 0, nsm = 0, resident[3] = {};
+  long long columns[3] = {};
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  for (int c = 0; c < 3; ++c) {
+    const void *fn = (c == 0)   ? (const void *)sweep2d_tma_batch_kernel<6>
+                     : (c == 1) ? (const void *)sweep2d_tma_batch_kernel<4>
+                                : (const void *)sweep2d_tma_batch_kernel<2>;
+    const int smem = (c == 0) ? (int)Cfg<6>::SMEM : (c == 1) ? (int)Cfg<4>::SMEM : (int)Cfg<2>::SMEM;
+    int per_sm = 0;
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NTHREADS, smem)) != cudaSuccess) return e;
+    resident[c] = nsm * std::max(per_sm, 1);
+    for (const ibdvm_ctx *ctx : cases)
+      if (ctx->oct_kc == 32 * kVpl[c]) columns[c] += (long long)((ctx->geom.n[0] + TX - 1) / TX) * (ctx->nvp / ctx->oct_kc);
+  }
   for (int i = 0; i < n; ++i) {
     const ibdvm_ctx *ctx = cases[i];
     if (ctx->oct_kc <= 0) return cudaErrorInvalidValue;
-    const int vpl = ctx->oct_kc / 32;
+    const int vpl = ctx->oct_kc / 32, cls = (vpl == 6) ? 0 : (vpl == 4) ? 1 : 2;
+    const bool whole = rows == 0 || (rows < 0 && columns[cls] >= (long long)kWholeItems * resident[cls]);
     for (int p = 0; p < 2; ++p) {
       const int cur = ctx->cur ^ p;
       args[2 * i + p] = oct2_args(ctx, cur, flags + i);
@@ -773,8 +799,7 @@ cudaError_t tma_batch_build(const std::vector<ibdvm_ctx *> &cases, const std::ve
     }
     // items: column strips x velocity chunks x row ranges of about `rows` rows
     const int nx = ctx->geom.n[0], ny = ctx->geom.n[1];
-    const int nrb = (rows < 0) ? std::max(1, (ny + kAutoRows / 2) / kAutoRows)
-                               : (rows == 0 || rows >= ny) ? 1 : (ny + rows - 1) / rows;
+    const int nrb = whole ? 1 : (rows < 0) ? std::max(1, (ny + kAutoRows / 2) / kAutoRows) : (ny + rows - 1) / rows;
     const int per = (ny + nrb - 1) / nrb;
     for (int x0 = 0; x0 < nx; x0 += TX)
       for (int c = 0; c < ctx->nvp / ctx->oct_kc; ++c)
@@ -795,13 +820,11 @@ cudaError_t tma_batch_build(const std::vector<ibdvm_ctx *> &cases, const std::ve
     if (a.vpl != b.vpl) return a.vpl > b.vpl;
     return (a.yb - a.ya) > (b.yb - b.ya);
   });
-  static const int kVpl[3] = {6, 4, 2};
   for (int c = 0, i = 0; c < 3; ++c) {
     t.cls_off[c] = i;
     while (i < static_cast<int>(items.size()) && items[i].vpl == kVpl[c]) ++i;
     t.cls_off[c + 1] = i;
   }
-  cudaError_t e;
   auto up = [&](const void *h, size_t bytes, void *&d) -> cudaError_t {
     cudaError_t r = cudaMalloc(&d, std::max<size_t>(bytes, 16));
     if (r != cudaSuccess || bytes == 0) return r;
@@ -814,22 +837,10 @@ cudaError_t tma_batch_build(const std::vector<ibdvm_ctx *> &cases, const std::ve
   if ((e = cudaMalloc(&nx, 3 * sizeof(int))) != cudaSuccess) return e;
   t.next = static_cast<int *>(nx);
   t.nitems = static_cast<int>(items.size());
-  int dev = 0, nsm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   t.grid = 0;
   for (int c = 0; c < 3; ++c) {
     const int n = t.cls_off[c + 1] - t.cls_off[c];
-    t.cls_grid[c] = 0;
-    if (n == 0) continue;
-    const void *fn = (c == 0)   ? (const void *)sweep2d_tma_batch_kernel<6>
-                     : (c == 1) ? (const void *)sweep2d_tma_batch_kernel<4>
-                                : (const void *)sweep2d_tma_batch_kernel<2>;
-    const int smem = (c == 0) ? (int)Cfg<6>::SMEM : (c == 1) ? (int)Cfg<4>::SMEM : (int)Cfg<2>::SMEM;
-    int per_sm = 0;
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NTHREADS, smem)) != cudaSuccess) return e;
-    t.cls_grid[c] = std::max(1, std::min(n, nsm * std::max(per_sm, 1)));
+    t.cls_grid[c] = (n == 0) ? 0 : std::min(n, resident[c]);
     t.grid = std::max(t.grid, t.cls_grid[c]);
   }
   return cudaStreamSynchronize(s); // the host tables go out of scope
