@@ -155,8 +155,9 @@ __device__ __forceinline__ double rcp_seed(double x) {
 
 // Downwind face f + ab / (a + b) for one-sided differences a, b of one sign,
 // else f (half the van Leer slope, Eq. limiter).  The sign and the range of
-// ab are read from its high word, off the FP64 pipe: a product below 2^-1022, an
-// infinite one or a NaN counts as no slope.  Called by whole warps.
+// ab are read from its high word, off the FP64 pipe: a product below 2^-1042 (a
+// subnormal number whose high word is zero), an infinite one or a NaN counts as no
+// slope.  Called by whole warps.
 __device__ __forceinline__ double face64(double f, double a, double b) {
   const double p = a * b;
   const bool slope = (unsigned)(__double2hiint(p) - 1) < 0x7fefffffu;
@@ -250,18 +251,15 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
       const double *fo = A.f + (size_t)(col0 + ps * p0) * A.nvp * NC;
       const int r = p0 - d;
       ijk[LA] = p0;
-      const double *fp = nullptr, *fpp = nullptr, *fd = nullptr;
-      unsigned mr = 0;
+      const double *fp = nullptr, *fpp = nullptr;
       const bool out = r < 0 || r >= nl;
       if (out) {
         fp = fpp = seen_row<D>(A, col0 + ps * p0, ijk, 0u, LA, -d);
       } else {
         const long long cr = col0 + ps * r;
-        mr = A.cmask[cr];
         ijk[LA] = r;
         fp = A.f + (size_t)cr * A.nvp * NC;
-        fpp = seen_row<D>(A, cr, ijk, mr, LA, -d);
-        if (!(mr & kNotFluidCell) && ((mr >> (2 * LA + (d > 0))) & 1u)) fd = seen_row<D>(A, cr, ijk, mr, LA, d);
+        fpp = seen_row<D>(A, cr, ijk, A.cmask[cr], LA, -d);
       }
 #pragma unroll
       for (int j = 0; j < KG; ++j)
@@ -270,21 +268,13 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
           ld<NC>(fo + (size_t)(kb + j) * NC, F[j]);
           ld<NC>(fp + (size_t)(kb + j) * NC, vp);
           ld<NC>(fpp + (size_t)(kb + j) * NC, vpp);
-          double vd[NC];
+          // a halo row has its value and no slope (vp - vpp is zero there); a ghost in
+          // row p0 takes no inflow, and the row after it replaces its own
 #pragma unroll
           for (int m = 0; m < NC; ++m) {
             Dd[j][m] = F[j][m] - vp[m];
-            vd[m] = Dd[j][m];
+            P[j][m] = face64(vp[m], vp[m] - vpp[m], Dd[j][m]);
           }
-          if (fd) {
-            double t[NC];
-            ld<NC>(fd + (size_t)(kb + j) * NC, t);
-#pragma unroll
-            for (int m = 0; m < NC; ++m) vd[m] = t[m] - vp[m];
-          }
-          // a halo row has its value and no slope (vp - vpp is zero there)
-#pragma unroll
-          for (int m = 0; m < NC; ++m) P[j][m] = face64(vp[m], vp[m] - vpp[m], vd[m]);
         }
     }
 
