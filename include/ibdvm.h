@@ -229,7 +229,8 @@ ibdvm_status ibdvm_set_body(ibdvm_ctx *ctx, const ibdvm_body_desc *body);
    Maxwellian at (T_w, U_w) (2D reduced: H_w = exp(-|xi - U_w|^2 / T_w) /
    (pi T_w), B_w = T_w / 2 H_w); for the other velocities they hold the
    boundary cell's own value, so the outgoing face value is the cell value;
-   rho_w (FP64, per boundary cell, from f^n each step) makes the mass flux
+   rho_w (per boundary cell, from f^n each step; FP64, in FP32 storage from sums
+   that keep the roundings of products and additions) makes the mass flux
    through the face zero, the velocities split by the plane xi_a = 0 (the
    lid-driven cavity of Sec. 4.1). */
 enum { IBDVM_FACE_FREESTREAM = 0, IBDVM_FACE_DIFFUSE_WALL = 1 };
@@ -240,9 +241,9 @@ typedef struct {
 } ibdvm_domain_desc;
 
 /* Sets the domain faces.  FP32 cases keep their TMA sweep, which reads the
-   wall halo at the domain faces; FP64 cases run the generic sweep kernel.
-   Cases with a wall cannot be batch members.  The state is kept.  With any wall the library allocates
-   (2 ncell / n[a] summed over the D axes) * nvel_padded * ncomp elements of
+   wall halo at the domain faces; FP64 cases keep the FP64 sweep, which reads it
+   as well.  Cases with a wall cannot be batch members.  The state is kept.  With
+   any wall the library allocates (2 ncell / n[a] summed over the D axes) * nvel_padded * ncomp elements of
    the storage type for the halo values and 6 nvel_padded doubles for the walls'
    Maxwellians, and frees them with the context or on the next call.
    Errors: IBDVM_E_INVAL (a bad kind, a z wall in 2D, T_w <= 0 or a

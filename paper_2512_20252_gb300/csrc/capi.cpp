@@ -411,7 +411,6 @@ void upload_body(ibdvm_ctx *ctx, const Geom *GV = nullptr, const std::vector<int
   ctx->nsc = static_cast<int>(nsc);
   ctx->nlink = static_cast<int>(nl);
   ctx->nghost = static_cast<int>(G.ghosts.size());
-  ctx->nsurf = static_cast<int>(ns);
   upload(ctx, ctx->dslot, dslot, "upload donor slots");
   upload(ctx, ctx->dlinks, dlinks, "upload donor links");
   upload(ctx, ctx->l_int, l_int, "upload link table");
@@ -1065,7 +1064,6 @@ ibdvm_status ibdvm_set_domain(ibdvm_ctx *ctx, const ibdvm_domain_desc *d) {
   for (int i = 0; i < 6; ++i) {
     ctx->wall_T[i] = (mask >> i & 1) ? d->T_w[i] : 1.0;
     ctx->wall_in[i] = in[i];
-    for (int a = 0; a < 3; ++a) ctx->wall_U[i][a] = (mask >> i & 1) ? d->U_w[i][a] : 0.0;
   }
   // the TMA sweeps read the wall halo at the domain faces
   ctx->use_tma = ctx->tma_ok;

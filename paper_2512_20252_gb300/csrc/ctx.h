@@ -109,18 +109,18 @@ struct ibdvm_ctx {
   // ghost band (its tables lie in one allocation)
   void *body_mem = nullptr;
   size_t body_bytes = 0;
-  int nlink = 0, nghost = 0, nsurf = 0;
+  int nlink = 0, nghost = 0;
   int *l_int = nullptr;      // [nlink][8]
   double *l_dbl = nullptr;   // [nlink][8]
   double *l_wg = nullptr;    // [nlink][nvp]
   double *l_cn = nullptr;    // [nlink][nvp] incident mass flux per unit f (ghost_tables_kernel)
   void *l_al = nullptr;      // [nlink][nvp] incident share of a velocity's box (FP32 storage)
   int *g_int = nullptr;      // [nghost][4]: first link, links, first and last + 1 surface entry
-  int *e_int = nullptr;      // [nsurf] surface cell of each entry
+  int *e_int = nullptr;      // surface cell of each entry of the ghosts' lists
   int *c_int = nullptr;      // [nsc][8]: cell, codes of its face neighbours
   int nsc = 0;               // distinct surface cells
   void *sig = nullptr;       // [nsc][dim][nvp][ncomp] their pre-ghost slopes
-  void *s_T = nullptr;       // [nsurf][8] in the storage type
+  void *s_T = nullptr;       // [entry][8] in the storage type
   void *lval = nullptr;      // [nlink][nvp][ncomp] ghost values f*_gc
   void *fi_scr = nullptr;    // [nlink][nvp][ncomp] incident distribution at the wall
   void *fsp_scr = nullptr;   // [nlink][nvp][ncomp] shifted-point value
@@ -152,7 +152,6 @@ struct ibdvm_ctx {
   // values [slots][nvp][ncomp] in the storage type
   int wall_mask = 0;
   double wall_T[6] = {1, 1, 1, 1, 1, 1};
-  double wall_U[6][3] = {};
   long long wall_off[7] = {};
   void *whalo = nullptr;
   // per face and stored velocity, the weight of the mass flux out of the

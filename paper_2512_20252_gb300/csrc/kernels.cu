@@ -1,8 +1,8 @@
 // kernels.cu -- CUDA kernels (sm_103a) of one forward-Euler step of the
 // ghost-cell immersed-boundary discrete velocity method (arXiv 2512.20252).
 //
-//   surface_slopes_kernel  the FP64 slopes of every surface entry, which the ghost
-//                       cells beside it share.
+//   surface_slopes_kernel  the pre-ghost slopes of every surface cell, in the storage
+//                       type, which the ghost cells beside it share.
 //   ghost_band_kernel   Sec. 3.2.1-3.2.3: per ghost cell, the upwind-weighted compact
 //                       interpolation f_gc (Eqs. extrapolation 1, upwind); per link, the
 //                       shifted point (Eqs. sp, fsp), the incident distribution
@@ -495,7 +495,8 @@ __device__ __forceinline__ void tree_upwind_face(const TreeStencil<T, NF> &S, T 
 }
 
 // FP64 storage, bound by its arithmetic (FP32 storage: tree_sweep.cu)
-template <typename T, int D> __global__ void __launch_bounds__(kBlock, 2) tree_sweep_kernel(TreeArgs<T> TA) {
+template <int D> __global__ void __launch_bounds__(kBlock, 2) tree_sweep_kernel(TreeArgs<double> TA) {
+  using T = double;
   constexpr int NC = Dims<D>::NC;
   constexpr int NM = Dims<D>::NM;
   constexpr int NF = 1 << (D - 1); // leaves at most beyond a face
@@ -1098,9 +1099,9 @@ template <typename T> struct GhostArgs {
   const double *__restrict__ l_cn;  // [nlink][nvp]: wg xn, the incident mass flux per unit f
   const T *__restrict__ l_al;       // [nlink][nvp], FP32 storage: wg / w, the incident share of a velocity's box
   const int *__restrict__ g_int;    // [nghost][4]: first link, links, first and last + 1 surface entry
-  const int *__restrict__ e_int;    // [nsurf]: the surface cell of an entry (index into c_int)
+  const int *__restrict__ e_int;    // [entry]: its surface cell (index into c_int)
   const int *__restrict__ c_int;    // [nsc][8]: surface cell, codes of its 6 face neighbours
-  const T *__restrict__ s_T;        // [nsurf][8]: r (weights), |r|, x_j - x_g, 1 / |r|
+  const T *__restrict__ s_T;        // [entry][8]: r (weights), |r|, x_j - x_g, 1 / |r|
   T *__restrict__ sig;              // [nsc][D][nvp][NC]: pre-ghost slopes of the surface cells
   const double *__restrict__ gwu;   // [nvp] unit-density wall Maxwellian
   const T *__restrict__ gwT;        // the same in FP32, FP32 storage
@@ -2039,19 +2040,17 @@ template <typename T, int D> cudaError_t sweep_t(ibdvm_ctx *ctx, int update, int
   return cudaGetLastError();
 }
 
-template <typename T, int D> cudaError_t tree_sweep_t(ibdvm_ctx *ctx) {
-  {
-    TreeArgs<T> A{};
-    A.S = sweep_args<T>(ctx, 1, 1);
-    A.sti = reinterpret_cast<const int4 *>(ctx->tree_sti);
-    A.stg = reinterpret_cast<const double2 *>(ctx->tree_stg);
-    A.lrec = reinterpret_cast<const int4 *>(ctx->tree_lrec);
-    A.sched = ctx->tree_sched;
-    dim3 block(kThreadsPerCell, kCellsPerBlock);
-    dim3 grid((unsigned)((ctx->ncell + kCellsPerBlock - 1) / kCellsPerBlock), (unsigned)ctx->nchunk);
-    tree_sweep_kernel<T, D><<<grid, block, 0, ctx->stream>>>(A);
-    return cudaGetLastError();
-  }
+template <int D> cudaError_t tree_sweep64_launch(ibdvm_ctx *ctx) {
+  TreeArgs<double> A{};
+  A.S = sweep_args<double>(ctx, 1, 1);
+  A.sti = reinterpret_cast<const int4 *>(ctx->tree_sti);
+  A.stg = reinterpret_cast<const double2 *>(ctx->tree_stg);
+  A.lrec = reinterpret_cast<const int4 *>(ctx->tree_lrec);
+  A.sched = ctx->tree_sched;
+  dim3 block(kThreadsPerCell, kCellsPerBlock);
+  dim3 grid((unsigned)((ctx->ncell + kCellsPerBlock - 1) / kCellsPerBlock), (unsigned)ctx->nchunk);
+  tree_sweep_kernel<D><<<grid, block, 0, ctx->stream>>>(A);
+  return cudaGetLastError();
 }
 
 // arguments of the finalize kernel for moment buffer parity wcur
@@ -2389,7 +2388,7 @@ cudaError_t launch_sweep(ibdvm_ctx *ctx) {
       if constexpr (std::is_same<T, double>::value) {
         const bool faces = !ctx->tree && ctx->plan64.nbatch > 0;
         ctx->kernel_launches[kKSweep] += faces ? sweep64_launches(ctx) : 1;
-        e = ctx->tree ? tree_sweep_t<T, D>(ctx) : faces ? sweep64_launch(ctx) : sweep_t<T, D>(ctx, 1, 1);
+        e = ctx->tree ? tree_sweep64_launch<D>(ctx) : faces ? sweep64_launch(ctx) : sweep_t<T, D>(ctx, 1, 1);
       } else {
         // (a tree: the regular leaves and the others)
         ctx->kernel_launches[kKSweep] += ctx->tree ? (ctx->tree_nreg > 0) + (ctx->tree_nreg < ctx->ncell) : 1;

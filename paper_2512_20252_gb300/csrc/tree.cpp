@@ -213,8 +213,8 @@ void build_tree_stencils(int D, const std::vector<int> &lev, const std::vector<i
 // The order in which the sweep's blocks take the leaves: within each window
 // of 256 consecutive leaves (the caller's order, near in space for leaves in
 // Z order), the regular leaves (the gather-first path), then the other fluid
-// leaves (the general path), then the solid ones, so that the four leaves of
-// a block take paths of about the same length while the blocks of a window
+// leaves (the general path), then the solid ones, so that the leaves of a block
+// (four in FP64, two in FP32) take paths of about the same length while the blocks of a window
 // share the rows they read.  split (the FP32 sweep, which launches the regular
 // leaves by themselves): all regular leaves first, then the others by window.
 std::vector<int> tree_schedule(int D, const std::vector<int> &lrec, bool split, int *nreg) {
