@@ -793,6 +793,8 @@ def measure_case(args, workload, world, rank, local, pg, with_cpu=True):
     sweep_ms, sweep_n = kt["sweep"]
     sweep_step_ms = sweep_ms / args.steps  # FP64 and tree sweeps take several launches a step
     kname, ksrc = SWEEP_KERNELS[int(info.sweep_variant), esize]
+    if kname == "sweep64_kernel" and sweep_n == args.steps:  # the smallest FP64 grids: no table launch
+        kname, ksrc = SWEEP_KERNELS[0, 4]
     alg_bytes = pairs * ncomp * esize * 2  # read f^n, write f^{n+1}
     peak, peak_kind = peaks()
     achieved = alg_bytes / (sweep_step_ms / 1e3) / 1e9 if sweep_n else None
@@ -828,9 +830,10 @@ def measure_case(args, workload, world, rank, local, pg, with_cpu=True):
                 "frac": (achieved / peak) if achieved else None,
                 "traffic": profiled_traffic(kname, ksrc, pairs, int(info.dim)),
                 "kernel": kname, "peak_kind": peak_kind,
-                "alg_bytes_per_launch": alg_bytes, "avg_launch_ms": sweep_step_ms}
+                "alg_bytes_per_launch": alg_bytes * args.steps / max(sweep_n, 1),
+                "avg_launch_ms": sweep_ms / max(sweep_n, 1), "sweep_ms_per_step": sweep_step_ms}
     fpp = (profiled_fp64_flops_per_pair(int(info.dim))
-           if args.precision == "fp64" and not case.get("tree") else None)
+           if kname == "sweep64_kernel" else None)
     if fpp and sweep_n:
         # the FP64 path is bound by GB300's FP64 arithmetic rate, not by HBM:
         # its roof is the FMA rate measured now on this GPU (clocks sampled)
@@ -844,7 +847,8 @@ def measure_case(args, workload, world, rank, local, pg, with_cpu=True):
                     "kernel": kname, "peak_kind": "measured FP64 FMA rate (ibdvm_fp64_fma_rate)",
                     "peak_clocks": peak_clocks, "peak_ms": peak_ms, "nominal_fp64_tflops": FP64_NOMINAL_TFLOPS,
                     "fp64_flops_per_pair": fpp,
-                    "hbm_achieved_gbs": achieved, "avg_launch_ms": sweep_step_ms}
+                    "hbm_achieved_gbs": achieved, "avg_launch_ms": sweep_ms / max(sweep_n, 1),
+                    "sweep_ms_per_step": sweep_step_ms}
     line = None
     if rank == 0:
         line = {
