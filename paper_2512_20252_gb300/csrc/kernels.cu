@@ -866,7 +866,7 @@ template <typename T, typename P = double> struct FinalArgs {
 // Cells (threads) of a finalize block.  The kernel is a chain of FP64 arithmetic
 // per cell (FP64 storage: a pow and a dozen divisions), so a small grid wants
 // many small blocks; the last block adds the residual sums.  Before, with blocks
-// of 256 and a kernel for the residual / now: 48^2 cells in FP64 39 / 33 us, 128^2 39 / 43,
+// of 256 and a kernel for the residual / now: 48^2 cells in FP64 39 / 31 us, 128^2 39 / 40,
 // octree of 46,584 leaves 52 / 37; FP32, 185 x 171 cells 35 / 31, 512^2 115 / 111, the
 // 64^3 sphere 249 / 245 (with products with 1 / rho for the divisions, which are less
 // exact, 262, and 101 at 512^2).  Kept out: four chunks' loads at a time (64^3: 466 us),
@@ -945,12 +945,14 @@ __device__ __forceinline__ void finalize_body(const FinalArgs<T, P> &A, const in
 #pragma unroll
         for (int m = 0; m < NM; ++m) low[m] = 0.0;
         for (int ch = 0; ch < A.nchunk; ch += 4, pc += 4 * st) {
+          // (beyond the last chunk: the first of the four read again, and not counted)
           const int n = A.nchunk - ch;
+          const size_t o1 = n > 1 ? st : 0, o2 = n > 2 ? 2 * st : 0, o3 = n > 3 ? 3 * st : 0;
 #pragma unroll
           for (int m = 0; m < NM; ++m) {
             const double *p = pc + (size_t)m * A.ncell;
-            const double p1 = n > 1 ? p[st] : 0.0, p2 = n > 2 ? p[2 * st] : 0.0, p3 = n > 3 ? p[3 * st] : 0.0;
-            const double y = ((p[0] + p1) + (p2 + p3)) - low[m], t = M[m] + y;
+            const double v0 = p[0], v1 = p[o1], v2 = p[o2], v3 = p[o3];
+            const double y = ((v0 + (n > 1 ? v1 : 0.0)) + ((n > 2 ? v2 : 0.0) + (n > 3 ? v3 : 0.0))) - low[m], t = M[m] + y;
             low[m] = (t - M[m]) - y;
             M[m] = t;
           }
