@@ -35,8 +35,8 @@
 //
 // Measured per step, tables included, on a state with slopes everywhere: 128^2
 // cells x 40^2 velocities between walls 3.12 ms (the sweep that formed every
-// face twice and divided took 9.55), 24^3 cells x 12^3 velocities 2.66 ms (7.48),
-// 48^2 x 24^2 0.193 ms (0.54).  3 to 4% of these go into roundings: f^{n+1} rounded
+// face twice and divided took 9.55), 24^3 cells x 12^3 velocities 2.60 ms (7.48),
+// 48^2 x 24^2 0.193 ms (0.54).  2 to 4% of these go into roundings: f^{n+1} rounded
 // once, compensated sums, the tables' exact products (without them the rms error
 // of f against extended precision was 1.2 to 1.4 times that of the sweep that
 // divided, of the sums up to 1.7 times; now 0.7 to 0.9 and 0.8 to 1.1).  Kept out, at
@@ -507,12 +507,13 @@ template <int D> __global__ void __launch_bounds__(32 * W64, 2) sweep64_kernel(S
         auto at = [&](int w) { return (D == 2) ? q[w * NM * 32] + q[w * NM * 32 + 16] : q[w * NM * 32]; };
         const double v = (at(0) + at(1)) + (at(2) + at(3));
         const double s = ar[e];
-        if (A.per > 2) {
+        const int m = e / CT; // (the second moments enter times the change of U only)
+        if (A.per > 2 && (m < D + 2 || m >= NM - D)) {
           const double y = v - __hiloint2double(lr[e], 0), t = s + y;
           lr[e] = __double2hiint((t - s) - y);
           ar[e] = t;
         } else {
-          ar[e] = s + v; // (two terms; the finalize kernel's sum over chunks is compensated)
+          ar[e] = s + v;
         }
       }
     }
