@@ -48,9 +48,9 @@ constexpr int kBlock = kThreadsPerCell * kCellsPerBlock;
 // velocities and adds the wall-density sums through distributed shared memory,
 // so that a body of few ghosts still spreads over the chip.  What bounds it is
 // the latency of the gathers (FP64 storage: the FP64 pipe's).  Per step, both
-// kernels: 64^3 sphere (144 ghosts, 312 links, 20^3 velocities) 221 us, where one
+// kernels: 64^3 sphere (144 ghosts, 312 links, 20^3 velocities) 200 us, where one
 // block of 512 threads per link, two rounds of them, had taken 867; octree sphere
-// (672 links) 398 us (1487); 24^3 sphere in FP64 124 us (791).  Threads per block, and the
+// (672 links) 346 us (1487); 24^3 sphere in FP64 126 us (791).  Threads per block, and the
 // velocities a block of the slope kernel takes.
 constexpr int kGhostSplit = 8;
 constexpr int kGhostThreads = 128;
@@ -1295,7 +1295,10 @@ __device__ __forceinline__ void mirrored(const GhostArgs<T> &G, const int l, con
 // f, weight and flux and get a zero ghost value): f_gc, which the links share,
 // then per link the shifted point, the incident distribution and, after the
 // cluster's sum for the wall density, the wall distribution and ghost value.
-template <typename T, int D> __device__ __forceinline__ void ghost_band_body(const GhostArgs<T> &G, const int g) {
+// SPEC: some links may reflect specularly (alpha < 1); without, the code for the
+// mirror images costs no registers.
+template <typename T, int D, bool SPEC>
+__device__ __forceinline__ void ghost_band_body(const GhostArgs<T> &G, const int g) {
   constexpr int NC = Dims<D>::NC;
   constexpr int NQ = 2 * D;                   // links of a ghost at most
   constexpr int NE = (D == 2) ? 8 : 26;       // surface cells of a ghost at most
@@ -1424,13 +1427,16 @@ template <typename T, int D> __device__ __forceinline__ void ghost_band_body(con
   double S[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) S[q] = 0.0;
-  if (alpha < 1.0) {
+  if (SPEC && alpha < 1.0) {
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
       if (q < nq) {
         const int l = l0 + q;
         const double nw[3] = {G.l_dbl[8 * l + 3], G.l_dbl[8 * l + 4], G.l_dbl[8 * l + 5]};
         for (int k = k0 + threadIdx.x; k < k1; k += kGhostThreads) {
+          // padding positions, most of a small 3D grid's, have no mirror image (with
+          // them 16^3 cells x 8^3 velocities took 159 us at alpha = 0.6, now 118)
+          if (!(G.wD[k] > 0.0)) continue;
           double xn, v[NC];
           mirrored<T, D>(G, l, k, nw, xn, v);
           S[q] += (G.wD[k] - G.l_wg[(size_t)l * G.nvp + k]) * xn * v[0];
@@ -1454,7 +1460,7 @@ template <typename T, int D> __device__ __forceinline__ void ghost_band_body(con
         double fsv[NC], xn;
 #pragma unroll
         for (int m = 0; m < NC; ++m) fsv[m] = 0.0;
-        if (alpha < 1.0) mirrored<T, D>(G, l, k, nw, xn, fsv);
+        if (SPEC && alpha < 1.0 && G.wD[k] > 0.0) mirrored<T, D>(G, l, k, nw, xn, fsv);
         const size_t o = ((size_t)l * G.nvp + k) * NC;
         T fi[NC], sp[NC], gv[NC];
         load_nc<T, NC>(G.fi + o, fi);
@@ -1518,9 +1524,9 @@ __global__ void __launch_bounds__(256) ghost_tables_kernel(GhostArgs<T> G, doubl
   if (threadIdx.x == 0) ld[7] = Dsum;
 }
 
-template <typename T, int D>
+template <typename T, int D, bool SPEC>
 __global__ void __launch_bounds__(kGhostThreads) ghost_band_kernel(const __grid_constant__ GhostArgs<T> G) {
-  ghost_band_body<T, D>(G, blockIdx.x / cooperative_groups::this_cluster().num_blocks());
+  ghost_band_body<T, D, SPEC>(G, blockIdx.x / cooperative_groups::this_cluster().num_blocks());
 }
 
 // a launch of the ghost band's kernels: clusters of `split` blocks
@@ -1932,7 +1938,7 @@ __global__ void __launch_bounds__(kGhostThreads)
   const int c = group_case(start, ncase, vg);
   if (threadIdx.x == 0) sG = tab[2 * c + par];
   __syncthreads();
-  ghost_band_body<T, D>(sG, vg - __ldg(start + c));
+  ghost_band_body<T, D, true>(sG, vg - __ldg(start + c));
 }
 
 template <typename T, int D>
@@ -2188,7 +2194,9 @@ template <typename T, int D> cudaError_t ghost_t(ibdvm_ctx *ctx, double *dbg) {
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  return launch_clusters(ghost_band_kernel<T, D>, ctx->nghost, ghost_split(ctx->nvp), ctx->stream, G);
+  const int split = ghost_split(ctx->nvp);
+  return G.accom < 1.0 ? launch_clusters(ghost_band_kernel<T, D, true>, ctx->nghost, split, ctx->stream, G)
+                       : launch_clusters(ghost_band_kernel<T, D, false>, ctx->nghost, split, ctx->stream, G);
 }
 
 // arguments of the force kernels for state buffer parity cur
