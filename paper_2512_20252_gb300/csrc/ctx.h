@@ -108,7 +108,7 @@ struct ibdvm_ctx {
   alignas(64) unsigned char tmap3[2][3][128]; // 3D: tile, x halo strip, y halo strip per buffer
   // ghost band (its tables lie in one allocation)
   void *body_mem = nullptr;
-  size_t body_bytes = 0;
+  size_t body_bytes = 0, body_cap = 0; // bytes in use, and allocated
   int nlink = 0, nghost = 0;
   int *l_int = nullptr;      // [nlink][8]
   double *l_dbl = nullptr;   // [nlink][8]
